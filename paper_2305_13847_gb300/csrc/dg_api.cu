@@ -213,6 +213,27 @@ RefData<double> scaled_ref64(int order, const double two_over_h[3]) {
             r.dliftm_s[j][a] = sc * sc * r.dliftm[a];
             r.dliftp_s[j][a] = sc * sc * r.dliftp[a];
         }
+    // exponents of the tables for the fixed-point contractions: |entry| < 2^q
+    auto above = [](const double *x, int n, int q0 = -1000) {
+        for (int i = 0; i < n; ++i)
+            if (x[i] != 0.0) q0 = std::max(q0, std::ilogb(x[i]) + 1);
+        return q0;
+    };
+    for (int j = 0; j < 3; ++j) {
+        const double sc = two_over_h[j];
+        double dm[36], dt[12];
+        for (int i = 0; i < 36; ++i) dm[i] = sc * r.dmat[i / 6][i % 6];
+        for (int i = 0; i < 6; ++i) {
+            dt[i] = sc * r.dlm[i];
+            dt[6 + i] = sc * r.dlp[i];
+        }
+        r.q_vol[j] = above(&r.dhat_s[j][0][0], 36);
+        r.q_lift[j] = above(r.liftp_s[j], 6, above(r.liftm_s[j], 6));
+        r.q_dlift[j] = above(r.dliftp_s[j], 6, above(r.dliftm_s[j], 6));
+        r.q_dmat[j] = above(dm, 36);
+        r.q_dtrace[j] = above(dt, 12);
+    }
+    r.q_trace = above(r.lp, 6, above(r.lm, 6));
     return r;
 }
 }  // namespace dgm
@@ -615,10 +636,9 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
         c->nf = c->L32->nf; c->np = c->L32->np; c->nfp1 = c->L32->nfp1;
         c->nd = c->L32->nd; c->ntr = c->L32->ntr; c->epb = c->L32->epb;
     } else {
-        if (g.precision == DG_FP64_FFC)
-            c->L64 = g.dim == 2 ? launchers_d2_f64ff(g.order, g.rain) : launchers_d3_f64ff(g.order, g.rain);
-        else
-            c->L64 = g.dim == 2 ? launchers_d2_f64(g.order, g.rain) : launchers_d3_f64(g.order, g.rain);
+        // DG_FP64_FFC is float64 too: its contractions run on the integer pipe
+        // with more bits than the float32 pairs of that form had
+        c->L64 = g.dim == 2 ? launchers_d2_f64(g.order, g.rain) : launchers_d3_f64(g.order, g.rain);
         c->LA = g.dim == 2 ? adj_launchers_d2(g.order, g.rain) : adj_launchers_d3(g.order, g.rain);
         c->nf = c->L64->nf; c->np = c->L64->np; c->nfp1 = c->L64->nfp1;
         c->nd = c->L64->nd; c->ntr = c->L64->ntr; c->epb = c->L64->epb;

@@ -128,6 +128,9 @@ struct RefData {
     Real dhat_s[3][6][6];
     Real liftm_s[3][6], liftp_s[3][6];    // (2/h_j) l_a(-+1)/w_a
     Real dliftm_s[3][6], dliftp_s[3][6];  // (2/h_j)^2 l_a'(-+1)/w_a
+    // float64 tables: |entry| < 2^q for the scaled tables dhat_s, lift*_s, dlift*_s,
+    // (2/h_j) dmat, (2/h_j) dl* and for l* (fixed-point contractions, dg_fixed.cuh)
+    int q_vol[3], q_lift[3], q_dlift[3], q_dmat[3], q_dtrace[3], q_trace;
 };
 
 template <typename Real>
@@ -190,14 +193,11 @@ __device__ __forceinline__ void add_fallout(const KArgs<Real> &A, bool top, int 
 // TT_: the threads a stage tile aims at, EPB = TT_ / NP elements (at least
 // one).  128 in 3-D: a warp that waits at a tile barrier holds up three
 // others, not seven (measured: float32 steps -5 % against 256).
-// FF_: float64 storage type with the stage kernel's volume and lift
-// contractions as compensated float32-pair sums (DG_FP64_FFC, dg_math.cuh)
-template <int D_, int K_, bool RAIN_, int TT_ = (D_ == 3 ? 128 : 256), bool FF_ = false>
+template <int D_, int K_, bool RAIN_, int TT_ = (D_ == 3 ? 128 : 256)>
 struct Shape {
     static constexpr int D = D_;
     static constexpr int K = K_;
     static constexpr bool RAIN = RAIN_;
-    static constexpr bool FF = FF_;
     static constexpr int P1 = K + 1;
     static constexpr int NP = ipow(P1, D);        // nodes per element
     static constexpr int NFP1 = ipow(P1, D - 1);  // points per face
@@ -249,146 +249,41 @@ __device__ __forceinline__ int face_q_vert(int j, int q) {
     return q / P1;                  // j = 0 or 1: remaining (., vertical)
 }
 
-// A CTA's copy of the mesh's scaled reference tables, per direction j:
-// dhat_s[j][a][0 .. P1) for each a, then liftm_s[j], liftp_s[j], dliftm_s[j],
-// dliftp_s[j].  A thread indexes them by its own a_j; in shared memory the
-// threads of a warp read their different entries in one access, where the
-// kernel-parameter bank serves one address at a time.  The float64 tile
-// reads them here (measured -1.4 % per step); the float32 tile, whose
-// shared-memory pipe is the busier one, from the parameter bank.
+// Nodal fluxes of a float32 tile: interleaved field pairs (2p, 2p + 1), the
+// last pair padded when n_f is odd, [D][(n_f + 1) / 2][STR][2], so that the
+// volume term runs on 64-bit shared loads and paired fmas (fma.rn.f32x2, each
+// lane the scalar fma).
 template <class S>
-struct Coef {
-    static constexpr int ROWS = S::P1 * S::P1;
-    static constexpr int LM = ROWS, LP = ROWS + S::P1, DLM = ROWS + 2 * S::P1, DLP = ROWS + 3 * S::P1;
-    static constexpr int BLK = (ROWS + 4 * S::P1 + 3) / 4 * 4;   // whole 16-byte groups (float)
-    static constexpr int N = S::D * BLK;
-};
-
-template <class S, typename Real>
-__device__ __forceinline__ void coef_fill(const RefData<Real> &r, Real *s_cf) {
-    using C = Coef<S>;
-    for (int i = threadIdx.x; i < C::N; i += blockDim.x) {
-        const int j = i / C::BLK, k = i - j * C::BLK;
-        Real v = Real(0);
-        if (k < C::LM) v = r.dhat_s[j][k / S::P1][k % S::P1];
-        else if (k < C::LP) v = r.liftm_s[j][k - C::LM];
-        else if (k < C::DLM) v = r.liftp_s[j][k - C::LP];
-        else if (k < C::DLP) v = r.dliftm_s[j][k - C::DLM];
-        else if (k < C::DLP + S::P1) v = r.dliftp_s[j][k - C::DLP];
-        s_cf[i] = v;
-    }
-}
-
-// Nodal-flux words per node and direction.  float32 stores the fields as
-// interleaved pairs (2p, 2p + 1), the last pair padded when n_f is odd,
-// [D][(n_f + 1) / 2][STR][2]: the volume term then runs on 64-bit shared
-// loads and paired fmas (fma.rn.f32x2, each lane the scalar fma).  float64
-// keeps [D][n_f][STR].
-template <class S, typename Real>
 __host__ __device__ constexpr int fl_words() {
-    return (sizeof(Real) == sizeof(float) || S::FF) ? 2 * ((S::NF + 1) / 2) : S::NF;
+    return 2 * ((S::NF + 1) / 2);
 }
 
 // index of field f of direction j at tile node t in the nodal fluxes
-template <class S, typename Real, int STR>
+template <class S, int STR>
 __device__ __forceinline__ int fl_index(int j, int f, int t) {
-    if constexpr (sizeof(Real) == sizeof(float))
-        return ((j * ((S::NF + 1) / 2) + (f >> 1)) * STR + t) * 2 + (f & 1);
-    else
-        return (j * S::NF + f) * STR + t;
+    return ((j * ((S::NF + 1) / 2) + (f >> 1)) * STR + t) * 2 + (f & 1);
 }
 
 // the fluxes F[0 .. n_f) of direction j at tile node t
-template <class S, typename Real, int STR>
-__device__ __forceinline__ void fl_store(Real *s_fl, int j, int t, const Real *F) {
-    if constexpr (sizeof(Real) == sizeof(float)) {
-        constexpr int NPR = (S::NF + 1) / 2;
-        float2 *fl2 = reinterpret_cast<float2 *>(s_fl);
+template <class S, int STR>
+__device__ __forceinline__ void fl_store(float *s_fl, int j, int t, const float *F) {
+    constexpr int NPR = (S::NF + 1) / 2;
+    float2 *fl2 = reinterpret_cast<float2 *>(s_fl);
 #pragma unroll
-        for (int p = 0; p < NPR; ++p)
-            fl2[(j * NPR + p) * STR + t] = make_float2(F[2 * p], 2 * p + 1 < S::NF ? F[2 * p + 1] : 0.0f);
-    } else {
-#pragma unroll
-        for (int f = 0; f < S::NF; ++f) s_fl[(j * S::NF + f) * STR + t] = F[f];
-    }
+    for (int p = 0; p < NPR; ++p)
+        fl2[(j * NPR + p) * STR + t] = make_float2(F[2 * p], 2 * p + 1 < S::NF ? F[2 * p + 1] : 0.0f);
 }
 
 // Volume term of Eq. (3.2), sum factorised, at node a of local element el:
 // R_a += sum_i dhat_s[j][a_j][i] F_j(line node i) for every direction j, from
-// the nodal fluxes s_fl [D][NF][STR]; coefficients from s_cf (Coef, float64)
-// or from the kernel arguments (float32)
-template <class S, typename Real, int STR>
-__device__ __forceinline__ void volume_term(const KArgs<Real> &A, const Real *s_fl,
-                                            const Real *s_cf, int el, int a, Real *R) {
-#pragma unroll
-    for (int j = 0; j < S::D; ++j) {
-        const int aj = digit<S::D, S::P1>(a, j);
-        const int st = stride_of<S::P1>(j);
-        const int b0 = el * S::NP + a - aj * st;
-        if constexpr (sizeof(Real) == sizeof(double)) {
-            Real c[S::P1];
-#pragma unroll
-            for (int i = 0; i < S::P1; ++i) c[i] = s_cf[j * Coef<S>::BLK + aj * S::P1 + i];
-#pragma unroll
-            for (int f = 0; f < S::NF; ++f) {
-                const Real *fl = s_fl + (j * S::NF + f) * STR + b0;
-                Real acc = R[f];
-#pragma unroll
-                for (int i = 0; i < S::P1; ++i) acc = fma(c[i], fl[i * st], acc);
-                R[f] = acc;
-            }
-        } else {
-            // field pairs: lane x is field 2p, lane y field 2p + 1, each the
-            // same fma chain as one field at a time
-            constexpr int NPR = (S::NF + 1) / 2;
-            const float2 *fl2 = reinterpret_cast<const float2 *>(s_fl);
-            float2 c[S::P1];
-#pragma unroll
-            for (int i = 0; i < S::P1; ++i) {
-                const float ci = A.ref.dhat_s[j][aj][i];
-                c[i] = make_float2(ci, ci);
-            }
-#pragma unroll
-            for (int p = 0; p < NPR; ++p) {
-                const float2 *fl = fl2 + (j * NPR + p) * STR + b0;
-                float2 acc = make_float2(R[2 * p], 2 * p + 1 < S::NF ? R[2 * p + 1] : 0.0f);
-#pragma unroll
-                for (int i = 0; i < S::P1; ++i) acc = __ffma2_rn(c[i], fl[i * st], acc);
-                R[2 * p] = acc.x;
-                if (2 * p + 1 < S::NF) R[2 * p + 1] = acc.y;
-            }
-        }
-    }
-}
-
-// ---- float-float contractions of the float64 form (DG_FP64_FFC) ----------
-// The coefficient tables of Coef as float32 pairs (ff_split of the float64
-// entries), in the same slots.
-template <class S>
-__device__ __forceinline__ void coef_fill_ff(const RefData<double> &r, float2 *s_cf) {
-    using C = Coef<S>;
-    for (int i = threadIdx.x; i < C::N; i += blockDim.x) {
-        const int j = i / C::BLK, k = i - j * C::BLK;
-        double v = 0.0;
-        if (k < C::LM) v = r.dhat_s[j][k / S::P1][k % S::P1];
-        else if (k < C::LP) v = r.liftm_s[j][k - C::LM];
-        else if (k < C::DLM) v = r.liftp_s[j][k - C::LP];
-        else if (k < C::DLP) v = r.dliftm_s[j][k - C::DLM];
-        else if (k < C::DLP + S::P1) v = r.dliftp_s[j][k - C::DLP];
-        s_cf[i] = ff_split(v);
-    }
-}
-
-// Volume term of Eq. (3.2) as in volume_term, every product and sum as a
-// compensated float32-pair operation, two fields at a time: (Rs, Re)[p] +=
-// sum_i dhat_s[j][a_j][i] F_j(line node i) for the fields 2p (lane x) and
-// 2p + 1 (lane y).  fl4 [D][(NF + 1) / 2][STR] holds (hi_2p, hi_2p+1, lo_2p,
-// lo_2p+1) per node, the coefficients are pairs (coef_fill_ff); the terms of
-// each field are taken in the float64 form's order.
+// the nodal fluxes s_fl (fl_store), coefficients from the kernel arguments.
+// Field pairs: lane x is field 2p, lane y field 2p + 1, each the same fma
+// chain as one field at a time.
 template <class S, int STR>
-__device__ __forceinline__ void volume_term_ff(const float4 *fl4, const float2 *cf2, int el, int a,
-                                               float2 *Rs, float2 *Re) {
+__device__ __forceinline__ void volume_term(const KArgs<float> &A, const float *s_fl, int el, int a,
+                                            float *R) {
     constexpr int NPR = (S::NF + 1) / 2;
+    const float2 *fl2 = reinterpret_cast<const float2 *>(s_fl);
 #pragma unroll
     for (int j = 0; j < S::D; ++j) {
         const int aj = digit<S::D, S::P1>(a, j);
@@ -396,45 +291,18 @@ __device__ __forceinline__ void volume_term_ff(const float4 *fl4, const float2 *
         const int b0 = el * S::NP + a - aj * st;
         float2 c[S::P1];
 #pragma unroll
-        for (int i = 0; i < S::P1; ++i) c[i] = cf2[j * Coef<S>::BLK + aj * S::P1 + i];
-#pragma unroll
-        for (int p = 0; p < NPR; ++p) {
-            const float4 *fl = fl4 + (j * NPR + p) * STR + b0;
-#pragma unroll
-            for (int i = 0; i < S::P1; ++i) {
-                const float4 x = fl[i * st];
-                ff_madd2(c[i], make_float2(x.x, x.y), make_float2(x.z, x.w), Rs[p], Re[p]);
-            }
+        for (int i = 0; i < S::P1; ++i) {
+            const float ci = A.ref.dhat_s[j][aj][i];
+            c[i] = make_float2(ci, ci);
         }
-    }
-}
-
-// Lift of the face fluxes (phase 3 of the stage tile) with float32 pairs, two
-// fields at a time: (Rs, Re) -= (2/h_j) l_a(+1)/w_a Fhat(j, +) and += (2/h_j)
-// l_a(-1)/w_a times the low face's value (the outward flux inline, G along
-// +e_j with the face pass, hence the sign), the high face first as in the
-// float64 form.  fh2 holds the face fluxes as (hi, lo) per field.
-template <class S, bool PF>
-__device__ __forceinline__ void lift_ff(const float2 *fh2, const float2 *cf2, int el, int a,
-                                        float2 *Rs, float2 *Re) {
-    constexpr int NPR = (S::NF + 1) / 2;
-#pragma unroll
-    for (int j = 0; j < S::D; ++j) {
-        const int aj = digit<S::D, S::P1>(a, j);
-        const int q = face_q<S::D, S::P1>(a, j);
-        const float2 *fm = fh2 + ((el * S::NFACE + 2 * j) * S::NF) * S::NFP1 + q;
-        const float2 *fp = fh2 + ((el * S::NFACE + 2 * j + 1) * S::NF) * S::NFP1 + q;
-        const float2 cm = cf2[j * Coef<S>::BLK + Coef<S>::LM + aj];
-        const float2 cp = ff_neg(cf2[j * Coef<S>::BLK + Coef<S>::LP + aj]);
-        const float2 cmo = PF ? cm : ff_neg(cm);
 #pragma unroll
         for (int p = 0; p < NPR; ++p) {
-            const bool two = 2 * p + 1 < S::NF;
-            const float2 p0 = fp[2 * p * S::NFP1], m0 = fm[2 * p * S::NFP1];
-            const float2 p1 = two ? fp[(2 * p + 1) * S::NFP1] : make_float2(0.0f, 0.0f);
-            const float2 m1 = two ? fm[(2 * p + 1) * S::NFP1] : make_float2(0.0f, 0.0f);
-            ff_madd2(cp, make_float2(p0.x, p1.x), make_float2(p0.y, p1.y), Rs[p], Re[p]);
-            ff_madd2(cmo, make_float2(m0.x, m1.x), make_float2(m0.y, m1.y), Rs[p], Re[p]);
+            const float2 *fl = fl2 + (j * NPR + p) * STR + b0;
+            float2 acc = make_float2(R[2 * p], 2 * p + 1 < S::NF ? R[2 * p + 1] : 0.0f);
+#pragma unroll
+            for (int i = 0; i < S::P1; ++i) acc = __ffma2_rn(c[i], fl[i * st], acc);
+            R[2 * p] = acc.x;
+            if (2 * p + 1 < S::NF) R[2 * p + 1] = acc.y;
         }
     }
 }
@@ -1185,8 +1053,8 @@ __device__ __forceinline__ void write_line(const KArgs<Real> &A, const RefData<R
     }
 }
 
-// One thread per face point: the float64 form, whose FP64 pipe is the bound,
-// runs faster with the trace work spread over more threads (measured).
+// One thread per face point, float64 sums: the float64 tile's path for values
+// outside its fixed-point range (dg_stage64.cuh).
 template <class S, typename Real, bool DIFF>
 __device__ __forceinline__ void write_traces_points(const KArgs<Real> &A, const RefData<Real> &ref,
                                                     const Real *s_tr, Real *trace_out, int bidx) {
@@ -1220,17 +1088,12 @@ __device__ __forceinline__ void write_traces_points(const KArgs<Real> &A, const 
     }
 }
 
-// Traces of the tile's state on all 2D faces.  float32: one thread per line
-// (both ends; the float32 tile is bound by instruction issue, and this halves
-// the shared-memory reads and index work, measured -22 % per step);
-// float64: one thread per face point (write_traces_points).
+// Traces of a float32 tile's state on all 2D faces, one thread per line (both
+// ends: the tile is bound by instruction issue, and this halves the
+// shared-memory reads and index work, measured -22 % per step).
 template <class S, typename Real, bool DIFF = false>
 __device__ __forceinline__ void write_traces(const KArgs<Real> &A, const RefData<Real> &ref,
                                              const Real *s_tr, Real *trace_out, int bidx) {
-    if (sizeof(Real) == sizeof(double)) {
-        write_traces_points<S, Real, DIFF>(A, ref, s_tr, trace_out, bidx);
-        return;
-    }
     const int ne = A.M.ne;
     for (int item = threadIdx.x; item < S::EPB * S::D * S::NFP1; item += S::NT) {
         const int el = item / (S::D * S::NFP1);
@@ -1390,18 +1253,17 @@ __device__ __forceinline__ NodeDerived derive_node(const float *u, const KArgs<f
                                       A.bnode[lev], A.bnode[nl + lev], A.M, A.rvs_tab, Tprev);
 }
 
-// STRIDE: nodes per field row of s_tr (0: the stage tile's EPB NP)
-template <class S, typename Real, bool DIFF = false, int STRIDE = 0>
-__device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real *u, int e, int a,
-                                                int iz, Real *s_tr, int t, Real *s_red = nullptr,
-                                                Real Tprev = Real(-1)) {
+// Split at one node: counts failures and stores the derived fields
+template <class S, typename Real>
+__device__ __forceinline__ void derive_and_store(const KArgs<Real> &A, const Real *u, int e, int a, int iz,
+                                                 Real Tprev, Real &T, Real &rv, Real &pp, Real &vr) {
     const size_t nodes = (size_t)A.M.ne * S::NP;
     const size_t gi = (size_t)e * S::NP + a;
     const int lev = iz * S::P1 + digit<S::D, S::P1>(a, S::VERT);
     const NodeDerived nd = derive_node<S>(u, A, lev, Tprev);
     if (!nd.conv) atomicAdd(&A.flags[0], 1ull);
     if (!nd.phys) atomicAdd(&A.flags[1], 1ull);
-    Real T, rv, pp, gm, vr;
+    Real gm;
     if (sizeof(Real) == sizeof(float)) {
         T = (Real)nd.Tf;
         rv = (Real)nd.rvf;
@@ -1422,7 +1284,19 @@ __device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real
         A.derived[3 * nodes + gi] = gm;
         A.derived[4 * nodes + gi] = vr;
     }
-    if (DIFF) alpha_accumulate<S, Real>(A, A.ref, u, vr, a, lev, s_red + 2 * (t / S::NP));
+}
+
+// The same, and the node values of the traces to s_tr.
+// STRIDE: nodes per field row of s_tr (0: the stage tile's EPB NP)
+template <class S, typename Real, bool DIFF = false, int STRIDE = 0>
+__device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real *u, int e, int a,
+                                                int iz, Real *s_tr, int t, Real *s_red = nullptr,
+                                                Real Tprev = Real(-1)) {
+    Real T, rv, pp, vr;
+    derive_and_store<S, Real>(A, u, e, a, iz, Tprev, T, rv, pp, vr);
+    if (DIFF)
+        alpha_accumulate<S, Real>(A, A.ref, u, vr, a, iz * S::P1 + digit<S::D, S::P1>(a, S::VERT),
+                                  s_red + 2 * (t / S::NP));
     const int str = STRIDE > 0 ? STRIDE : S::EPB * S::NP;
 #pragma unroll
     for (int f = 0; f < S::NF; ++f) s_tr[f * str + t] = u[f];
@@ -1431,7 +1305,21 @@ __device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real
     s_tr[(S::NF + 2) * str + t] = pp;
 }
 
+// Eq. (3.8) at a node at the end of a step: relax rho_m', rho_r', m, E' towards
+// 0 by dl and add the moisture removed to rho_d' (Section 3.6)
+template <class S, typename Real>
+__device__ __forceinline__ void apply_sponge(Real dl, Real *un) {
+    if (dl == Real(0)) return;
+    const Real om = Real(1) - dl;
+    Real removed = dl * un[1];
+    if (S::RAIN) removed = add_rn(removed, dl * un[2]);
+    un[0] = un[0] + removed;
+#pragma unroll
+    for (int f = 1; f < S::NF; ++f) un[f] = om * un[f];
+}
+
 // DIFF: also the element coefficients alpha_K and the derivative traces
+// (float32; the float64 tile's is k_prepare64, dg_stage64.cuh)
 template <class S, typename Real, bool DIFF>
 __global__ void __launch_bounds__(S::NT) k_prepare(KArgs<Real> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1465,43 +1353,35 @@ __global__ void __launch_bounds__(S::NT) k_prepare(KArgs<Real> A) {
 constexpr int MODE_RHS = 0;
 constexpr int MODE_STAGE = 1;
 
-// Shared memory of a stage tile: nodal fluxes s_fl (fl_index), node
+// Shared memory of a float32 stage tile: nodal fluxes s_fl (fl_index), node
 // values for the traces s_tr [NTR][EPB NP], outward face fluxes s_fh
 // [EPB][2D][NFP][NFP1] (with diffusion NFP = 2 NF: the fluxes, then the
 // symmetry terms), per-element indices, with diffusion the element's vertex
-// coefficients [EPB][2][2^D] and its alpha sums [EPB][2], and (float64) the
-// coefficient tables s_cf (Coef).  s_tr is needed before the volume phase
-// only when the float32 inline form interpolates its own traces in the face
-// phase, or with diffusion (the derivatives of the node values); otherwise
-// it is filled after the volume phase and shares s_fl.
-template <class S, typename Real, bool PF, bool DIFF = false>
+// coefficients [EPB][2][2^D] and its alpha sums [EPB][2].  s_tr is needed
+// before the volume phase only when the inline form interpolates its own
+// traces in the face phase, or with diffusion (the derivatives of the node
+// values); otherwise it is filled after the volume phase and shares s_fl.
+template <bool PF, bool DIFF = false>
 __host__ __device__ constexpr bool tr_shares_fl() {
-    return (PF || sizeof(Real) == sizeof(double)) && !DIFF;
+    return PF && !DIFF;
 }
 
 // byte offset of s_fh (16-byte aligned for the asynchronous copy of the face fluxes)
 template <class S, typename Real, bool PF, bool DIFF>
 __host__ __device__ constexpr size_t stage_fh_offset() {
-    constexpr size_t FL = (size_t)S::D * fl_words<S, Real>();
-    return ((sizeof(Real) * (tr_shares_fl<S, Real, PF, DIFF>()
+    constexpr size_t FL = (size_t)S::D * fl_words<S>();
+    return ((sizeof(Real) * (tr_shares_fl<PF, DIFF>()
                                  ? (FL > (size_t)S::NTR ? FL : (size_t)S::NTR)
                                  : FL + S::NTR) *
              S::EPB * S::NP) + 15) / 16 * 16;
 }
 
-// byte offset of the coefficient tables s_cf (Coef; 16-byte aligned)
-template <class S, typename Real, bool PF, bool DIFF>
-__host__ __device__ constexpr size_t stage_cf_offset() {
+template <class S, typename Real, bool PF = false, bool DIFF = false>
+constexpr size_t stage_smem_bytes() {
     constexpr size_t fh = (size_t)S::EPB * S::NFACE * (DIFF ? 2 * S::NF : S::NF) * S::NFP1;
     return (stage_fh_offset<S, Real, PF, DIFF>() + sizeof(Real) * fh +
             sizeof(int) * 16 * (size_t)S::EPB +  // per element: 2D neighbours, vertical index
             (DIFF ? sizeof(Real) * (size_t)S::EPB * (2 * S::NCORNER + 2) : 0) + 15) / 16 * 16;
-}
-
-template <class S, typename Real, bool PF = false, bool DIFF = false>
-constexpr size_t stage_smem_bytes() {
-    return stage_cf_offset<S, Real, PF, DIFF>() +
-           (sizeof(Real) == sizeof(double) ? sizeof(Real) * (size_t)Coef<S>::N : 0);
 }
 
 // completes the asynchronous copies issued by this thread
@@ -1817,7 +1697,7 @@ __global__ void __launch_bounds__(kFaceThreads) k_face(KArgs<Real> A) {
     }
 }
 
-// One tile of EPB consecutive elements (tile index bidx) of the stage
+// One float32 tile of EPB consecutive elements (tile index bidx) of the stage
 // kernel; every thread of the CTA takes part (the body has barriers).
 // PF: the face fluxes come from the face pass (k_face) instead of being
 // evaluated here on both sides of every face.
@@ -1826,21 +1706,15 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
                                             unsigned char *smem_raw) {
     static_assert(!DIFF || PF, "artificial diffusion runs with the face pass");
     constexpr int STR = S::EPB * S::NP;
-    constexpr bool SHARE = tr_shares_fl<S, Real, PF, DIFF>();
+    constexpr bool SHARE = tr_shares_fl<PF, DIFF>();
     constexpr int NFP = DIFF ? 2 * S::NF : S::NF;             // per face: fluxes [, symmetry terms]
     constexpr int EB = S::NFACE * NFP * S::NFP1;              // face values of one element
-    // float64 form with float-float contractions: nodal fluxes, coefficient
-    // tables and face fluxes held as float32 pairs in the float64 slots, the
-    // tendencies accumulated as pairs (Rs, Re) through the volume term and the
-    // lift, then formed in float64 for the stage update
-    constexpr bool FFC = S::FF && sizeof(Real) == sizeof(double) && !DIFF;
     Real *s_fl = reinterpret_cast<Real *>(smem_raw);          // nodal fluxes (fl_index)
-    Real *s_tr = SHARE ? s_fl : s_fl + S::D * fl_words<S, Real>() * STR;   // [NTR][STR]
+    Real *s_tr = SHARE ? s_fl : s_fl + S::D * fl_words<S>() * STR;   // [NTR][STR]
     Real *s_fh = reinterpret_cast<Real *>(smem_raw + stage_fh_offset<S, Real, PF, DIFF>());  // [EPB][EB]
     int *s_info = reinterpret_cast<int *>(s_fh + S::EPB * EB);                            // [EPB][16]
     Real *s_al = reinterpret_cast<Real *>(s_info + 16 * S::EPB);        // DIFF: [EPB][2][NCORNER]
     Real *s_red = s_al + S::EPB * 2 * S::NCORNER;                       // DIFF: [EPB][2]
-    Real *s_cf = reinterpret_cast<Real *>(smem_raw + stage_cf_offset<S, Real, PF, DIFF>());
     const MeshData &M = A.M;
     const int ne = M.ne;
     const size_t nodes = (size_t)ne * S::NP;
@@ -1868,11 +1742,6 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
     // face pass: copy the tile's face values to shared memory while the
     // nodal phases run (one contiguous block per face)
     if (PF) cp_async_faces<S, Real, NFP>(A.fbuf, A.ftab, s_fh, bidx, min(S::EPB, ne - bidx * S::EPB));
-
-    if constexpr (FFC)
-        coef_fill_ff<S>(A.ref, reinterpret_cast<float2 *>(s_cf));
-    else if (sizeof(Real) == sizeof(double))
-        coef_fill<S, Real>(A.ref, s_cf);
 
     // per element: neighbours across the 2D faces (inline faces) and the
     // vertical index
@@ -1911,30 +1780,16 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
         for (int j = 0; j < S::D; ++j) {
             Real F[S::NF];
             flux_dir<S, Real>(P, j, F);
-            if constexpr (FFC) {
-                // (hi, hi, lo, lo) of the field pairs (2p, 2p + 1), the last
-                // padded with zeros when n_f is odd
-                constexpr int NPR = (S::NF + 1) / 2;
-                float4 *fl4 = reinterpret_cast<float4 *>(s_fl);
-#pragma unroll
-                for (int p = 0; p < NPR; ++p) {
-                    const float2 v0 = ff_split(to_f64(F[2 * p]));
-                    const float2 v1 =
-                        2 * p + 1 < S::NF ? ff_split(to_f64(F[2 * p + 1])) : make_float2(0.0f, 0.0f);
-                    fl4[(j * NPR + p) * STR + t] = make_float4(v0.x, v1.x, v0.y, v1.y);
-                }
-            } else {
-                fl_store<S, Real, STR>(s_fl, j, t, F);
-            }
+            fl_store<S, STR>(s_fl, j, t, F);
         }
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) R[f] = Real(0);
-        // node values for the own traces (the float64 form reads them back
-        // from the trace buffer) or for the derivatives of the diffusion
+        // node values for the own traces (inline faces) or for the
+        // derivatives of the diffusion
         if (DIFF) {
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) s_tr[f * STR + t] = u[f];
-        } else if (!PF && sizeof(Real) == sizeof(float)) {
+        } else if (!PF) {
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) s_tr[f * STR + t] = u[f];
             s_tr[S::NF * STR + t] = T;
@@ -1974,7 +1829,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
 #pragma unroll
                     for (int i = 0; i < S::P1; ++i) du = fma(ref.dmat[aj][i], v[i * st], du);
                     const Real al = (S::RAIN && f == 2) ? ar : au;
-                    s_fl[fl_index<S, Real, STR>(j, f, t)] -= al * (sc * du);
+                    s_fl[fl_index<S, STR>(j, f, t)] -= al * (sc * du);
                 }
             }
         }
@@ -1982,24 +1837,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
     }
 
     // ---- phase 2a: volume term, sum factorised: R_a += (2/h_j) sum_i dhat[a_j][i] F_j(i)
-    constexpr int NPR = (S::NF + 1) / 2;
-    float2 Rs[NPR], Re[NPR];     // FFC: the tendencies of the field pairs (2p, 2p + 1)
-    if constexpr (FFC) {
-        if (valid) {
-#pragma unroll
-            for (int p = 0; p < NPR; ++p) {
-                const float2 r0 = ff_split(to_f64(R[2 * p]));
-                const float2 r1 =
-                    2 * p + 1 < S::NF ? ff_split(to_f64(R[2 * p + 1])) : make_float2(0.0f, 0.0f);
-                Rs[p] = make_float2(r0.x, r1.x);
-                Re[p] = make_float2(r0.y, r1.y);
-            }
-            volume_term_ff<S, STR>(reinterpret_cast<const float4 *>(s_fl),
-                                   reinterpret_cast<const float2 *>(s_cf), el, a, Rs, Re);
-        }
-    } else {
-        if (valid) volume_term<S, Real, STR>(A, s_fl, s_cf, el, a, R);
-    }
+    if (valid) volume_term<S, STR>(A, s_fl, el, a, R);
 
     // ---- phase 2b: Lax-Friedrichs flux at every face point of the CTA's elements
     if (PF) {
@@ -2031,39 +1869,16 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
         }
     }
     __syncthreads();
-    if constexpr (FFC) {
-        // the tile's face fluxes as float32 pairs, in place (each thread
-        // rewrites the slots it reads)
-        const int nv = min(S::EPB, ne - bidx * S::EPB) * EB;
-        float2 *fh2 = reinterpret_cast<float2 *>(s_fh);
-        for (int i = t; i < nv; i += S::NT) fh2[i] = ff_split(to_f64(s_fh[i]));
-        __syncthreads();
-    }
 
     // ---- phase 3: lift the face fluxes, R_a -= (2/h_j) l_a(s)/w_a Fhat(j, s)
     if (valid) {
-        if constexpr (FFC) {
-            lift_ff<S, PF>(reinterpret_cast<const float2 *>(s_fh), reinterpret_cast<const float2 *>(s_cf),
-                           el, a, Rs, Re);
 #pragma unroll
-            for (int f = 0; f < S::NF; ++f)
-                R[f] = (f & 1) ? ff_value(Rs[f >> 1].y, Re[f >> 1].y) : ff_value(Rs[f >> 1].x, Re[f >> 1].x);
-        }
-#pragma unroll
-        for (int j = 0; j < (FFC ? 0 : S::D); ++j) {
+        for (int j = 0; j < S::D; ++j) {
             const int aj = digit<S::D, S::P1>(a, j);
             const int q = face_q<S::D, S::P1>(a, j);
             const Real *fm = s_fh + ((el * S::NFACE + 2 * j) * NFP) * S::NFP1 + q;
             const Real *fp = s_fh + ((el * S::NFACE + 2 * j + 1) * NFP) * S::NFP1 + q;
-            const Real *cf = s_cf + j * Coef<S>::BLK;
-            Real cm, cp;
-            if constexpr (sizeof(Real) == sizeof(double)) {
-                cm = cf[Coef<S>::LM + aj];
-                cp = cf[Coef<S>::LP + aj];
-            } else {
-                cm = A.ref.liftm_s[j][aj];
-                cp = A.ref.liftp_s[j][aj];
-            }
+            const Real cm = A.ref.liftm_s[j][aj], cp = A.ref.liftp_s[j][aj];
             // the low face holds the outward flux (inline) or G along +e_j,
             // which is minus this element's outward flux (face pass):
             // fma(-c, -G, r) = fma(c, G, r) exactly, so both schedules round
@@ -2077,14 +1892,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
                 // symmetry term of Eq. (3.7): + (2/h_j)^2 l_a'(s)/w_a S on both faces
                 const Real *sm = fm + S::NF * S::NFP1;
                 const Real *sp = fp + S::NF * S::NFP1;
-                Real dm, dp;
-                if constexpr (sizeof(Real) == sizeof(double)) {
-                    dm = cf[Coef<S>::DLM + aj];
-                    dp = cf[Coef<S>::DLP + aj];
-                } else {
-                    dm = A.ref.dliftm_s[j][aj];
-                    dp = A.ref.dliftp_s[j][aj];
-                }
+                const Real dm = A.ref.dliftm_s[j][aj], dp = A.ref.dliftp_s[j][aj];
 #pragma unroll
                 for (int f = 0; f < S::NF; ++f)
                     R[f] = fma(dm, sm[f * S::NFP1], fma(dp, sp[f * S::NFP1], R[f]));
@@ -2104,19 +1912,9 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
                 if (nonzero(A.alpha)) v = fma(A.alpha, A.Un[f * nodes + gi], v);
                 un[f] = v;
             }
-            if (A.sponge) {
-                // Eq. (3.8) at the end of the step: relax rho_m', rho_r', m, E'
-                // towards 0 and add the moisture removed to rho_d' (Section 3.6)
-                const Real dl = A.sponge[s_info[el * 16 + 6] * S::P1 + digit<S::D, S::P1>(a, S::VERT)];
-                if (dl != Real(0)) {
-                    const Real om = Real(1) - dl;
-                    Real removed = dl * un[1];
-                    if (S::RAIN) removed = add_rn(removed, dl * un[2]);
-                    un[0] = un[0] + removed;
-#pragma unroll
-                    for (int f = 1; f < S::NF; ++f) un[f] = om * un[f];
-                }
-            }
+            if (A.sponge)
+                apply_sponge<S, Real>(
+                    A.sponge[s_info[el * 16 + 6] * S::P1 + digit<S::D, S::P1>(a, S::VERT)], un);
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) A.Uout[f * nodes + gi] = un[f];
             split_and_store<S, Real, DIFF>(A, un, e, a, s_info[el * 16 + 6], s_tr, t, s_red, dT);

@@ -7,13 +7,13 @@
 
 #include "dg_column.cuh"
 #include "dg_device.cuh"
+#include "dg_stage64.cuh"
 
 namespace dgm {
 
 template <typename Real>
 struct Launchers {
     int nf, np, nfp1, nd, ntr, epb, nt;
-    size_t prep_smem, stage_smem;
     // diff: with the artificial diffusion of Eq. (3.7) (face pass only)
     cudaError_t (*prepare)(const KArgs<Real> &, bool diff, cudaStream_t);
     // pf: the stage kernel takes its face fluxes from the face pass
@@ -38,24 +38,40 @@ inline int grid_for(size_t n, int threads) {
 
 template <class S, typename Real>
 struct Impl {
-    static constexpr size_t prep_smem = sizeof(Real) * ((size_t)S::NTR * S::EPB * S::NP + 2 * S::EPB);
-    static constexpr size_t stage_smem = stage_smem_bytes<S, Real, false>();
-    static constexpr size_t stage_smem_pf = stage_smem_bytes<S, Real, true>();
-    static constexpr size_t stage_smem_diff = stage_smem_bytes<S, Real, true, true>();
+    static constexpr bool F64 = std::is_same<Real, double>::value;
+
+    // shared memory of the prepare and stage tiles
+    template <bool DIFF>
+    static constexpr size_t prep_smem() {
+        if constexpr (F64) return prepare64_smem_bytes<S, DIFF>();
+        else return sizeof(Real) * ((size_t)S::NTR * S::EPB * S::NP + 2 * S::EPB);
+    }
+    template <bool PF, bool DIFF>
+    static constexpr size_t stage_smem() {
+        if constexpr (F64) return stage64_smem_bytes<S, DIFF>();
+        else return stage_smem_bytes<S, Real, PF, DIFF>();
+    }
 
     static int blocks(const KArgs<Real> &A) { return (A.M.ne + S::EPB - 1) / S::EPB; }
 
     template <bool DIFF>
+    static constexpr auto prepare_kernel() {
+        if constexpr (F64) return &k_prepare64<S, DIFF>;
+        else return &k_prepare<S, Real, DIFF>;
+    }
+
+    template <bool DIFF>
     static cudaError_t launch_prepare(const KArgs<Real> &A, cudaStream_t st) {
+        constexpr size_t smem = prep_smem<DIFF>();
+        const auto kern = prepare_kernel<DIFF>();
         static bool attr = false;
         if (!attr) {
-            cudaError_t err = cudaFuncSetAttribute(k_prepare<S, Real, DIFF>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)prep_smem);
+            cudaError_t err =
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (err != cudaSuccess) return err;
             attr = true;
         }
-        k_prepare<S, Real, DIFF><<<A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, prep_smem, st>>>(A);
+        kern<<<A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st>>>(A);
         return cudaGetLastError();
     }
 
@@ -67,8 +83,9 @@ struct Impl {
     // or 256 threads take the variant with the 48-register budget
     template <int MODE, bool PF, bool DIFF>
     static constexpr auto stage_kernel() {
-        if constexpr (std::is_same<Real, float>::value && PF && !DIFF &&
-                      (S::NT == 64 || S::NT == 128 || S::NT == 256))
+        if constexpr (F64)
+            return &k_stage64<S, MODE, PF, DIFF>;
+        else if constexpr (PF && !DIFF && (S::NT == 64 || S::NT == 128 || S::NT == 256))
             return &k_stage_f32pf<S, MODE>;
         else
             return &k_stage<S, Real, MODE, PF, DIFF>;
@@ -76,7 +93,7 @@ struct Impl {
 
     template <int MODE, bool PF, bool DIFF>
     static cudaError_t launch_stage(const KArgs<Real> &A, cudaStream_t st) {
-        constexpr size_t smem = DIFF ? stage_smem_diff : (PF ? stage_smem_pf : stage_smem);
+        constexpr size_t smem = stage_smem<PF, DIFF>();
         const auto kern = stage_kernel<MODE, PF, DIFF>();
         static bool attr = false;
         if (!attr) {
@@ -166,8 +183,6 @@ struct Impl {
         L.ntr = S::NTR;
         L.epb = S::EPB;
         L.nt = S::NT;
-        L.prep_smem = prep_smem;
-        L.stage_smem = stage_smem;
         L.prepare = &prepare;
         L.stage = &stage;
         L.face = &face;
@@ -175,7 +190,7 @@ struct Impl {
         L.split = &split;
         L.init_bubble = &init_bubble;
         L.reduce = &reduce;
-        if constexpr (std::is_same<Real, float>::value)
+        if constexpr (!F64)
             L.column = &column;
         else
             L.column = nullptr;
@@ -190,9 +205,6 @@ const Launchers<float> *launchers_d2_f32(int K, int rain);
 const Launchers<float> *launchers_d3_f32(int K, int rain);
 // float64 reference tables with the coefficients scaled by 2/h_j (dg_api.cu)
 RefData<double> scaled_ref64(int order, const double two_over_h[3]);
-// float64 with float-float contractions (DG_FP64_FFC)
-const Launchers<double> *launchers_d2_f64ff(int K, int rain);
-const Launchers<double> *launchers_d3_f64ff(int K, int rain);
 
 }  // namespace dgm
 
@@ -205,27 +217,6 @@ const Launchers<double> *launchers_d3_f64ff(int K, int rain);
             {Impl<Shape<DIM, 3, false>, REAL>::table(), Impl<Shape<DIM, 3, true>, REAL>::table()}, \
             {Impl<Shape<DIM, 4, false>, REAL>::table(), Impl<Shape<DIM, 4, true>, REAL>::table()}, \
             {Impl<Shape<DIM, 5, false>, REAL>::table(), Impl<Shape<DIM, 5, true>, REAL>::table()}, \
-        };                                                                             \
-        if (K < 1 || K > 5) return nullptr;                                            \
-        return &t[K - 1][rain ? 1 : 0];                                                \
-    }                                                                                  \
-    }
-
-#define DGM_FF_SHAPE(DIM, K, RAIN) Shape<DIM, K, RAIN, (DIM == 3 ? 128 : 256), true>
-#define DGM_DEFINE_LAUNCHERS_FF(NAME, DIM)                                             \
-    namespace dgm {                                                                    \
-    const Launchers<double> *NAME(int K, int rain) {                                   \
-        static const Launchers<double> t[5][2] = {                                     \
-            {Impl<DGM_FF_SHAPE(DIM, 1, false), double>::table(),                       \
-             Impl<DGM_FF_SHAPE(DIM, 1, true), double>::table()},                       \
-            {Impl<DGM_FF_SHAPE(DIM, 2, false), double>::table(),                       \
-             Impl<DGM_FF_SHAPE(DIM, 2, true), double>::table()},                       \
-            {Impl<DGM_FF_SHAPE(DIM, 3, false), double>::table(),                       \
-             Impl<DGM_FF_SHAPE(DIM, 3, true), double>::table()},                       \
-            {Impl<DGM_FF_SHAPE(DIM, 4, false), double>::table(),                       \
-             Impl<DGM_FF_SHAPE(DIM, 4, true), double>::table()},                       \
-            {Impl<DGM_FF_SHAPE(DIM, 5, false), double>::table(),                       \
-             Impl<DGM_FF_SHAPE(DIM, 5, true), double>::table()},                       \
         };                                                                             \
         if (K < 1 || K > 5) return nullptr;                                            \
         return &t[K - 1][rain ? 1 : 0];                                                \
