@@ -302,21 +302,23 @@ int copy_chunk(dg_ctx *c, int k, void *dst, const void *src, cudaMemcpyKind kind
 
 // split and traces of state U into trace buffer tb; ntiles > 0: only the
 // element tiles [tile0, tile0 + ntiles)
+// keep_rv: the derived fields hold rho_v for the adjoint kernels
 template <typename Real>
 int do_prepare(dg_ctx *c, const Launchers<Real> *L, const RefData<Real> &ref, const void *U, int tb,
-               int tile0, int ntiles) {
+               int tile0, int ntiles, bool keep_rv) {
     KArgs<Real> A = base_args<Real>(c, ref);
     A.Uin = (const Real *)U;
     A.trace_out = (Real *)c->trace[tb];
     A.dtrace_out = (Real *)c->dtrace[tb];
     A.tile0 = tile0;
     A.ntiles = ntiles;
+    A.keep_rv = keep_rv;
     return cuda_status(L->prepare(A, c->diff, c->stream));
 }
 
-int prepare(dg_ctx *c, const void *U, int tb, int tile0 = 0, int ntiles = 0) {
-    return c->fp32 ? do_prepare<float>(c, c->L32, c->ref32, U, tb, tile0, ntiles)
-                   : do_prepare<double>(c, c->L64, c->ref64, U, tb, tile0, ntiles);
+int prepare(dg_ctx *c, const void *U, int tb, int tile0 = 0, int ntiles = 0, bool keep_rv = false) {
+    return c->fp32 ? do_prepare<float>(c, c->L32, c->ref32, U, tb, tile0, ntiles, keep_rv)
+                   : do_prepare<double>(c, c->L64, c->ref64, U, tb, tile0, ntiles, keep_rv);
 }
 
 // Upload of a host state in kChunks chunks of whole element tiles: the
@@ -560,7 +562,7 @@ AdjArgs adj_args(const dg_ctx *c, const void *U, const double *w, double *out, d
 int rhs_adjoint_into(dg_ctx *c, const void *U, const double *w, double *out, double alpha,
                      double beta, double gamma) {
     c->derived_valid = false;
-    int st = prepare(c, U, 0);
+    int st = prepare(c, U, 0, 0, 0, true);
     if (st != DG_OK) return st;
     AdjArgs A = adj_args(c, U, w, out, alpha, beta, gamma);
     if (c->LA->local(A, c->stream) != cudaSuccess) return DG_ECUDA;
@@ -1137,7 +1139,7 @@ int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     if (!c->base_set) return DG_ESTATE;
     DeviceGuard dg(c->device);
     c->derived_valid = false;
-    int st = prepare(c, U, 0);
+    int st = prepare(c, U, 0, 0, 0, true);
     if (st != DG_OK) return st;
     AdjArgs A = adj_args(c, U, nullptr, dJdU, 0.0, 0.0, 1.0);
     if (c->LA->cloud(A, c->partials, c->nred, c->stream) != cudaSuccess) return DG_ECUDA;

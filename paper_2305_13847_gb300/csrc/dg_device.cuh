@@ -140,7 +140,7 @@ struct KArgs {
     const Real *Uin;       // state the operator is evaluated on (ABI layout)
     const Real *Un;        // U^n for the stage combination (may equal Uin)
     Real *Uout;            // MODE_RHS: dU/dt; MODE_STAGE: new stage state
-    Real *derived;         // [ND][nodes]
+    Real *derived;         // [ND][nodes]: T, rho_v (float64: 1/rho, see keep_rv), p' [, G_rm, v_r]
     const Real *trace_in;  // traces of Uin:   [2D][NTR][ne][NFP1]
     Real *trace_out;       // traces of Uout (MODE_STAGE)
     const Real *bnode;     // base at node levels [4][nzlev_node]: rho_d, rho_m, E, p
@@ -169,6 +169,7 @@ struct KArgs {
     // (ntiles 0: all), so that an upload is split while its chunks arrive
     // and a download starts while the last stage still runs
     int tile0, ntiles;
+    int keep_rv;           // float64 k_prepare: derived field 1 is rho_v (adjoint), else 1/rho
 };
 
 // float64 value of a storage-type value (widen: integer pipe)
@@ -506,18 +507,24 @@ __device__ __forceinline__ SplitResult split_point(double rd, double rm, double 
         const double lat = fma(kCvv - kCl, t0 - kTref, kLprime);
         const double h = fma(heat, t0 - kTref, fma(rvs, kLprime, -re));
         const double dh = fma(lat, drvs, heat);
-        const double d = -h * recip(dh);
-        if (abs_le(d, 3e-4)) {
+        // d = -H/H': the float32 quotient d0 and the float32 quotient of its
+        // float64 residual H + H' d0, together within 2^-44 of d (|d| <= 3e-4 K,
+        // so 2e-17 K); two float64 operations instead of a reciprocal's and a
+        // product's four
+        const float ridh = __frcp_rn(narrow(dh));
+        const float df = -narrow(h) * ridh;
+        if (fabsf(df) <= 3e-4f) {
+            const double d0 = widen(df);
+            const float d1 = -narrow(fma(dh, d0, h)) * ridh;
             // H'' = 2 (c_vv - c_l) rho_vs' + (c_vv - c_l)(T - T_ref) + L') rho_vs'',
             // rho_vs'' = rho_vs (phi1^2 + phi1'), phi1' = -(a-1)/T^2 - 2b/T^3
             const float itf = __frcp_rn(tf ? t : narrow(t0)), rvf = narrow(rvs);
             const float p1f = itf * (am1 + bb * itf);               // (ln rho_vs)
             const float d2rvs = rvf * (p1f * p1f - itf * itf * (am1 + 2.0f * bb * itf));
             const float d2h = 2.0f * clv * (rvf * p1f) + narrow(lat) * d2rvs;
-            const float df = narrow(d);
-            const float c2 = -0.5f * d2h / narrow(dh) * df * df;   // second-order term of the step
-            const double dc = d + widen(c2);
-            const float dcf = narrow(dc);
+            const float c2 = fmaf(-0.5f * d2h * ridh * df, df, d1);   // and the step's second-order term
+            const double dc = d0 + widen(c2);
+            const float dcf = df + c2;
             r.T = t0 + dc;
             r.rv = fma(drvs, dc, rvs) + widen(0.5f * d2rvs * dcf * dcf);
             r.converged = true;
@@ -574,6 +581,7 @@ __device__ __forceinline__ float rain_velocity(float rr, float rm, const MeshDat
 // Per-node split plus the node-local quantities the next operator needs.
 struct NodeDerived {
     double T, rv, pp, gm, vr;
+    double irho;                    // 1/rho (float64 form)
     float Tf, rvf, ppf, gmf, vrf;   // float32 copies (FP32-bulk form)
     float rcf;                      // rho_m - rho_v, perturbation form only
     bool conv, phys;
@@ -585,7 +593,8 @@ __device__ __forceinline__ NodeDerived node_derived(double rd, double rm, double
                                                     const double *__restrict__ tab) {
     NodeDerived o;
     const double rho = rd + rm + rr;
-    const double re = E - 0.5 * msq * recip(rho);
+    o.irho = recip(rho);
+    const double re = E - 0.5 * msq * o.irho;
     const SplitResult s = split_point<RAIN>(rd, rm, rr, re, tab, M.newton_cap);
     o.T = s.T;
     o.rv = s.rv;
@@ -596,20 +605,24 @@ __device__ __forceinline__ NodeDerived node_derived(double rd, double rm, double
     o.vr = 0.0;
     if (RAIN) {
         // Eq. (2.4): the rain powers from x = max(rho_r, 0)^(1/16) = r y^15, y = r^(-1/16)
+        // x^8 = r y^8, x^14 = r y^2, x^4 = r y^12, x^2 = x^4 y^2, x^3 = x^4 y; a saturated
+        // node has no evaporation (deficit 0) and an unsaturated one no cloud
         const bool rpos = gt0(rr);
-        const double rrp = rpos ? rr : 0.0;
-        double x = 0.0;
+        double y = 0.0, y2 = 0.0, x8 = 0.0, x4 = 0.0;
         if (rpos) {
-            const double y = inv_root16(rrp);
-            const double y2 = y * y, y4 = y2 * y2, y8 = y4 * y4;
-            x = rrp * (y8 * y4 * y2 * y);
+            y = inv_root16(rr);
+            y2 = y * y;
+            const double y4 = y2 * y2;
+            x8 = rr * (y4 * y4);
+            x4 = x8 * y4;
         }
-        const double x2 = x * x, x3 = x2 * x, x4 = x2 * x2, x8 = x4 * x4, x14 = x8 * x4 * x2;
+        const double x2 = x4 * y2;
+        if (nonzero(s.deficit)) {
+            const double x3 = x4 * y;
+            o.gm = (kSevA - kSevB * (s.T - kTref)) * fma(kSevC, x3, 1.0) * (s.deficit * x8);
+        }
         const double rc = rm - s.rv;
-        const double s_ev = (kSevA - kSevB * (s.T - kTref)) * (1.0 + kSevC * x3) * s.deficit * x8;
-        const double s_au = kSau * (gt0(rc) ? rc : 0.0);
-        const double s_ac = kSac * rc * x14;
-        o.gm = s_ev - s_au - s_ac;
+        if (nonzero(rc)) o.gm -= fma(kSac, rc * (rr * y2), gt0(rc) ? kSau * rc : 0.0);
         // v_r = kvr (rho_r / rho_w)^(1/8) = kvr x^2 rho_w^(-1/8) (Section 2.1)
         const double rw = gt0(M.rho_w) ? M.rho_w : rm + rr;
         o.vr = (rpos && gt0(rw)) ? M.kvr * x2 * inv_root8(rw) : 0.0;
@@ -921,14 +934,15 @@ struct Prim {
     Real m[D], u[D];
 };
 
+// inv: 1/rho
 template <class S, typename Real>
-__device__ __forceinline__ void make_prim(Prim<S::D, S::RAIN, Real> &P, const Real *U, Real brd,
-                                          Real brm, Real bE, Real bp, Real T, Real rv, Real pp) {
+__device__ __forceinline__ void make_prim_inv(Prim<S::D, S::RAIN, Real> &P, const Real *U, Real brd,
+                                              Real brm, Real bE, Real bp, Real T, Real rv, Real pp,
+                                              Real inv) {
     P.rd = brd + U[0];
     P.rm = brm + U[1];
     P.rr = S::RAIN ? U[2] : Real(0);
     P.rho = P.rd + P.rm + P.rr;
-    const Real inv = recip(P.rho);
     P.irho = inv;
 #pragma unroll
     for (int j = 0; j < S::D; ++j) {
@@ -941,6 +955,13 @@ __device__ __forceinline__ void make_prim(Prim<S::D, S::RAIN, Real> &P, const Re
     P.T = T;
     P.rv = rv;
     P.vr = Real(0);
+}
+
+template <class S, typename Real>
+__device__ __forceinline__ void make_prim(Prim<S::D, S::RAIN, Real> &P, const Real *U, Real brd,
+                                          Real brm, Real bE, Real bp, Real T, Real rv, Real pp) {
+    const Real rho = (brd + U[0]) + (brm + U[1]) + (S::RAIN ? U[2] : Real(0));
+    make_prim_inv<S, Real>(P, U, brd, brm, bE, bp, T, rv, pp, recip(rho));
 }
 
 // F_j(U): rho_d u_j, rho_m u_j, rho_r (u_j - v_r d_jz), m_i u_j - rho_r v_r u_i d_jz + p' d_ij,
@@ -974,10 +995,10 @@ __device__ __forceinline__ void flux_dir(const Prim<S::D, S::RAIN, Real> &P, int
 // (c_v, R per unit volume: c_vd rho_d + c_vv rho_v + c_l (rho_c + rho_r), R_d rho_d + R_v rho_v)
 template <class S, int J, typename Real>
 __device__ __forceinline__ Real wave_speed(const Prim<S::D, S::RAIN, Real> &P) {
-    const Real rc = P.rm - P.rv;
-    const Real cv = Real(kCvd) * P.rd + Real(kCvv) * P.rv + Real(kCl) * (rc + P.rr);
+    // c_l (rho_c + rho_r) + c_vv rho_v with rho_c = rho_m - rho_v
+    const Real cv = fma(Real(kCvd), P.rd, fma(Real(kCvv - kCl), P.rv, Real(kCl) * (P.rm + P.rr)));
     // c_m = sqrt(num / den) = num / sqrt(num den): one reciprocal square root
-    const Real num = (cv + Real(kRd) * P.rd + Real(kRv) * P.rv) * P.p;
+    const Real num = fma(Real(kRd), P.rd, fma(Real(kRv), P.rv, cv)) * P.p;
     const Real nd = num * (cv * P.rho);
     Real lam = fabs(P.u[J]) + (gt0(nd) ? num * rsqrt_nr(nd) : Real(0));
     if (S::RAIN && J == S::VERT) lam += fabs(P.vr);
@@ -1278,7 +1299,12 @@ __device__ __forceinline__ void derive_and_store(const KArgs<Real> &A, const Rea
         vr = (Real)nd.vr;
     }
     A.derived[gi] = T;
-    A.derived[nodes + gi] = rv;
+    // the float64 stage kernel's nodal flux takes 1/rho, which the split has
+    // formed, and not rho_v (its traces carry that); the adjoint takes rho_v
+    if (sizeof(Real) == sizeof(double))
+        A.derived[nodes + gi] = A.keep_rv ? rv : (Real)nd.irho;
+    else
+        A.derived[nodes + gi] = rv;
     A.derived[2 * nodes + gi] = pp;
     if (S::RAIN) {
         A.derived[3 * nodes + gi] = gm;
@@ -1436,6 +1462,72 @@ __device__ __forceinline__ void load_base(const Real *tab, int nlev, int lev, Re
     p = tab[3 * nlev + lev];
 }
 
+// ---------------------------------------------------------------------------
+// Face pass: the Lax-Friedrichs flux of Section 3.2 once per face point
+// ---------------------------------------------------------------------------
+// G = {{F_J}} + Lambda/2 (U_lo - U_hi) along +e_J at one face point from the
+// traces tl (element at the lower coordinate) and th (upper) and the base
+// state at the point.  Every schedule evaluates it with the same two sides in
+// the same order, so the inline schedule's outward fluxes are +G and -G
+// exactly.  The average is formed on half velocities, one product and one fma
+// per transported field (the two fluxes and their sum would take four
+// operations): with w = u_J / 2 (and w_r = w - v_r / 2 for rain, q =
+// rho_r v_r / 2 on faces normal to e_z)
+//   {{rho u}} = rho_h w_h + rho_l w_l, {{m_i u}} likewise - q u_i, + {{p'}} d_iJ,
+//   {{(E + p) u}} - (c_l (T - T_ref) + |u|^2/2) q.
+template <class S, typename Real, int J>
+__device__ __forceinline__ void lf_flux(const Real *tl, const Real *th, Real brd, Real brm, Real bE,
+                                        Real bp, const MeshData &M, Real *G) {
+    Prim<S::D, S::RAIN, Real> Pl, Ph;
+    make_prim<S, Real>(Pl, tl, brd, brm, bE, bp, tl[S::NF], tl[S::NF + 1], tl[S::NF + 2]);
+    make_prim<S, Real>(Ph, th, brd, brm, bE, bp, th[S::NF], th[S::NF + 1], th[S::NF + 2]);
+    constexpr bool FALL = S::RAIN && J == S::VERT;
+    if (FALL) {
+        Pl.vr = rain_velocity(Pl.rr, Pl.rm, M);
+        Ph.vr = rain_velocity(Ph.rr, Ph.rm, M);
+    }
+    const Real half = Real(0.5);
+    const Real wl = half * Pl.u[J], wh = half * Ph.u[J];
+    G[0] = fma(Ph.rd, wh, Pl.rd * wl);
+    G[1] = fma(Ph.rm, wh, Pl.rm * wl);
+    Real ql = Real(0), qh = Real(0);
+    if (S::RAIN) {
+        Real vl = wl, vh = wh;
+        if (FALL) {
+            ql = half * Pl.vr;
+            qh = half * Ph.vr;
+            vl -= ql;
+            vh -= qh;
+            ql *= Pl.rr;
+            qh *= Ph.rr;
+        }
+        G[2] = fma(Ph.rr, vh, Pl.rr * vl);
+    }
+#pragma unroll
+    for (int i = 0; i < S::D; ++i) {
+        Real g = fma(Ph.m[i], wh, Pl.m[i] * wl);
+        if (FALL) g = fma(-qh, Ph.u[i], fma(-ql, Pl.u[i], g));
+        if (i == J) g = fma(half, add_rn(Pl.pp, Ph.pp), g);
+        G[S::IM + i] = g;
+    }
+    Real ge = fma(Ph.E + Ph.p, wh, (Pl.E + Pl.p) * wl);
+    if (FALL) {
+        Real kl = Real(0), kh = Real(0);
+#pragma unroll
+        for (int i = 0; i < S::D; ++i) {
+            kl = fma(Pl.u[i], Pl.u[i], kl);
+            kh = fma(Ph.u[i], Ph.u[i], kh);
+        }
+        ge = fma(-qh, fma(Real(kCl), Ph.T - Real(kTref), half * kh), ge);
+        ge = fma(-ql, fma(Real(kCl), Pl.T - Real(kTref), half * kl), ge);
+    }
+    G[S::IE] = ge;
+    const Real ll = wave_speed<S, J, Real>(Pl), lh = wave_speed<S, J, Real>(Ph);
+    const Real hl = half * max_nonneg(ll, lh);
+#pragma unroll
+    for (int fld = 0; fld < S::NF; ++fld) G[fld] = fma(hl, tl[fld] - th[fld], G[fld]);
+}
+
 // Lax-Friedrichs flux F_n = {{F}}.n + Lambda/2 [[U]] (Section 3.2) at face point q of
 // face (J, s) of element e2, in the outward direction s e_J; own trace from
 // shared memory, neighbour trace from the trace buffer, slip-wall ghost state
@@ -1482,60 +1574,26 @@ __device__ __forceinline__ void face_point(const KArgs<Real> &A, const RefData<R
         load_base<S, Real>(A.bnode, M.nzlev_node, iz * S::P1 + face_q_vert<S::D, S::P1>(J, q), brd,
                            brm, bE, bp);
     }
-    Prim<S::D, S::RAIN, Real> Pm, Pp;
-    make_prim<S, Real>(Pm, tm, brd, brm, bE, bp, tm[S::NF], tm[S::NF + 1], tm[S::NF + 2]);
-    make_prim<S, Real>(Pp, tp, brd, brm, bE, bp, tp[S::NF], tp[S::NF + 1], tp[S::NF + 2]);
-    if (S::RAIN) {
-        Pm.vr = rain_velocity(Pm.rr, Pm.rm, M);
-        Pp.vr = rain_velocity(Pp.rr, Pp.rm, M);
+    // G along +e_J as in the face pass (so both schedules round identically),
+    // then the outward sign
+    Real G[S::NF], o[S::NF];
+#pragma unroll
+    for (int fld = 0; fld < S::NTR; ++fld) {
+        const Real lo = s > 0 ? tm[fld] : tp[fld];
+        tp[fld] = s > 0 ? tp[fld] : tm[fld];
+        tm[fld] = lo;
     }
-    Real Fm[S::NF], Fp[S::NF];
-    flux_dir<S, Real>(Pm, J, Fm);
-    flux_dir<S, Real>(Pp, J, Fp);
-    const Real lm = wave_speed<S, J, Real>(Pm), lpp = wave_speed<S, J, Real>(Pp);
-    const Real lam = max_nonneg(lm, lpp);
-    const Real hs = Real(0.5) * Real(s), hl = Real(0.5) * lam;
+    lf_flux<S, Real, J>(tm, tp, brd, brm, bE, bp, M, G);
     Real *out = s_fh + ((el2 * S::NFACE + face) * S::NF) * S::NFP1 + q;
-    // one explicit fma, as in face_flux: both schedules round identically
-    Real o[S::NF];
 #pragma unroll
     for (int f = 0; f < S::NF; ++f) {
-        o[f] = fma(hs, add_rn(Fm[f], Fp[f]), hl * (tm[f] - tp[f]));
+        o[f] = s > 0 ? G[f] : -G[f];
         out[f * S::NFP1] = o[f];
     }
     if (S::RAIN && J == S::VERT && nb < 0 && A.fallout) {
         const int nh = S::D == 3 ? M.n[0] * M.n[1] : M.n[0];
         add_fallout<S, Real>(A, s > 0, e2 % nh, q, to_f64(o[1]) + to_f64(o[2]));
     }
-}
-
-// ---------------------------------------------------------------------------
-// Face pass: the Lax-Friedrichs flux of Section 3.2 once per face point
-// ---------------------------------------------------------------------------
-// G = {{F_J}} + Lambda/2 (U_lo - U_hi) along +e_J at one face point from the
-// traces tl (element at the lower coordinate) and th (upper) and the base
-// state at the point.  The sum F_lo + F_hi is an unfused add and G one
-// explicit fma, so G does not depend on which side evaluates it, and the
-// inline schedule's outward fluxes are +G and -G exactly.
-template <class S, typename Real, int J>
-__device__ __forceinline__ void lf_flux(const Real *tl, const Real *th, Real brd, Real brm, Real bE,
-                                        Real bp, const MeshData &M, Real *G) {
-    Prim<S::D, S::RAIN, Real> Pl, Ph;
-    make_prim<S, Real>(Pl, tl, brd, brm, bE, bp, tl[S::NF], tl[S::NF + 1], tl[S::NF + 2]);
-    make_prim<S, Real>(Ph, th, brd, brm, bE, bp, th[S::NF], th[S::NF + 1], th[S::NF + 2]);
-    if (S::RAIN) {
-        Pl.vr = rain_velocity(Pl.rr, Pl.rm, M);
-        Ph.vr = rain_velocity(Ph.rr, Ph.rm, M);
-    }
-    Real Fl[S::NF], Fh[S::NF];
-    flux_dir<S, Real>(Pl, J, Fl);
-    flux_dir<S, Real>(Ph, J, Fh);
-    const Real ll = wave_speed<S, J, Real>(Pl), lh = wave_speed<S, J, Real>(Ph);
-    const Real lam = max_nonneg(ll, lh);
-    const Real hl = Real(0.5) * lam;
-#pragma unroll
-    for (int fld = 0; fld < S::NF; ++fld)
-        G[fld] = fma(Real(0.5), add_rn(Fl[fld], Fh[fld]), hl * (tl[fld] - th[fld]));
 }
 
 // G = {{F_j}} + Lambda/2 (U_lo - U_hi) along +e_j from the traces of the two

@@ -16,7 +16,7 @@
 // * r^(-1/n) from a float32 estimate by one third-order step
 //   y <- y (1 + e/n + (n+1) e^2/(2 n^2)), e = 1 - r y^n, which needs no
 //   division and reaches float64 rounding from the estimate's ~3e-7.
-// * Reciprocal and reciprocal square root by Newton-Raphson refinement of the
+// * Reciprocal and reciprocal square root by one third-order step from the
 //   hardware's approximate float64 reciprocal and reciprocal square root
 //   (measured against exact values: recip within 1 ulp, rsqrt_nr within 2,
 //   sqrt_nr within 3).
@@ -109,21 +109,21 @@ __device__ __forceinline__ double rsqrt_seed(double x) {
     return r;
 }
 
-// 1/x: two Newton-Raphson steps r <- r + r (1 - x r) from the seed
+// 1/x: one third-order step r <- r (1 + e + e^2), e = 1 - x r, from the
+// seed (three float64 operations, where two Newton steps take four; the
+// seed's ~1e-6 leaves e^3 ~ 1e-18)
 __device__ __forceinline__ double recip(double x) {
-    double r = rcp_seed(x);
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double r = rcp_seed(x);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
-// 1/sqrt(x): two Newton steps y <- y (3 - x y^2) / 2 from the seed
+// 1/sqrt(x): one third-order step y <- y (1 + e/2 + 3 e^2/8), e = 1 - x y^2,
+// from the seed (five float64 operations, where two Newton steps take seven)
 __device__ __forceinline__ double rsqrt_nr(double x) {
-    double y = rsqrt_seed(x);
-    double h = 0.5 * x;
-    y = y * fma(-h * y, y, 1.5);
-    return y * fma(-h * y, y, 1.5);
+    const double y = rsqrt_seed(x);
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 __device__ __forceinline__ double sqrt_nr(double x) { return x > 0.0 ? x * rsqrt_nr(x) : 0.0; }
@@ -141,33 +141,32 @@ __device__ __forceinline__ double sqrt_nr(double x) { return x > 0.0 ? x * rsqrt
 // smallest subnormal is 2^-1074 > 2^-96 2^-1152); the loop stops there also
 // for r <= 0, which the callers exclude (the result is then not a number).
 // r > 0 orders like its bit pattern, so the test needs no float64 compare.
+// 2^k, -1023 < k < 1024
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
 constexpr double kTiny = 0x1p-96;
 constexpr double kUp = 0x1p128;
 
 __device__ __forceinline__ double inv_root16(double r) {
-    double sc = 1.0;
-    for (int it = 0; it < 9 && __double_as_longlong(r) < __double_as_longlong(kTiny); ++it) {
-        r *= kUp;
-        sc *= 0x1p8;
-    }
+    int k = 0;       // scalings
+    for (; k < 9 && __double_as_longlong(r) < __double_as_longlong(kTiny); ++k) r *= kUp;
     const double y = widen(exp2f(-0.0625f * __log2f(narrow(r))));
     const double y2 = y * y, y4 = y2 * y2, y8 = y4 * y4;
     const double e = fma(-r, y8 * y8, 1.0);
     const double c = fma(17.0 / 512.0, e, 0.0625);
-    return fma(y * c, e, y) * sc;
+    const double v = fma(y * c, e, y);
+    return k == 0 ? v : v * pow2(8 * k);
 }
 
 __device__ __forceinline__ double inv_root8(double r) {
-    double sc = 1.0;
-    for (int it = 0; it < 9 && __double_as_longlong(r) < __double_as_longlong(kTiny); ++it) {
-        r *= kUp;
-        sc *= 0x1p16;
-    }
+    int k = 0;       // scalings
+    for (; k < 9 && __double_as_longlong(r) < __double_as_longlong(kTiny); ++k) r *= kUp;
     const double y = widen(exp2f(-0.125f * __log2f(narrow(r))));
     const double y2 = y * y, y4 = y2 * y2;
     const double e = fma(-r, y4 * y4, 1.0);
     const double c = fma(9.0 / 128.0, e, 0.125);
-    return fma(y * c, e, y) * sc;
+    const double v = fma(y * c, e, y);
+    return k == 0 ? v : v * pow2(16 * k);
 }
 
 // ---------------------------------------------------------------------------

@@ -263,6 +263,33 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
     if (DIFF) alpha_store<S, double>(A, s_red, bidx);
 }
 
+// F_j of flux_dir (dg_device.cuh) for every direction at a node; m_i u_j is
+// formed once for both orders of its indices.
+template <class S>
+__device__ __forceinline__ void flux_all(const Prim<S::D, S::RAIN, double> &P, double (*F)[S::NF]) {
+    double q = 0.0, e = P.E + P.p;
+    if (S::RAIN) q = P.rr * P.vr;
+#pragma unroll
+    for (int j = 0; j < S::D; ++j) {
+        F[j][0] = P.rd * P.u[j];
+        F[j][1] = P.rm * P.u[j];
+        if (S::RAIN) F[j][2] = j == S::VERT ? fma(P.rr, P.u[j], -q) : P.rr * P.u[j];
+        F[j][S::IM + j] = fma(P.m[j], P.u[j], P.pp);
+#pragma unroll
+        for (int i = 0; i < j; ++i) F[j][S::IM + i] = F[i][S::IM + j] = P.m[i] * P.u[j];
+        F[j][S::IE] = e * P.u[j];
+    }
+    if (S::RAIN) {
+        double ke = 0.0;
+#pragma unroll
+        for (int i = 0; i < S::D; ++i) {
+            ke = fma(P.u[i], P.u[i], ke);
+            F[S::VERT][S::IM + i] = fma(-q, P.u[i], F[S::VERT][S::IM + i]);
+        }
+        F[S::VERT][S::IE] = fma(-q, fma(kCl, P.T - kTref, 0.5 * ke), F[S::VERT][S::IE]);
+    }
+}
+
 // One tile of EPB consecutive elements (tile index bidx) of the stage kernel:
 // stage_block's phases (dg_device.cuh) with fixed-point contractions.  Every
 // thread of the CTA takes part.
@@ -296,12 +323,12 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
 
     // the node's state and derived fields: loads issued first, so that their
     // latency overlaps the set-up below
-    double u[S::NF], dT = 0.0, drv = 0.0, dpp = 0.0, dgm = 0.0, dvr = 0.0;
+    double u[S::NF], dT = 0.0, dir = 1.0, dpp = 0.0, dgm = 0.0, dvr = 0.0;
     if (valid) {
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) u[f] = A.Uin[f * nodes + gi];
         dT = A.derived[gi];
-        drv = A.derived[nodes + gi];
+        dir = A.derived[nodes + gi];
         dpp = A.derived[2 * nodes + gi];
         if (S::RAIN) {
             dgm = A.derived[3 * nodes + gi];
@@ -337,18 +364,17 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
         double brd, brm, bE, bp;
         load_base<S, double>(A.bnode, M.nzlev_node, lev, brd, brm, bE, bp);
         Prim<S::D, S::RAIN, double> P;
-        make_prim<S, double>(P, u, brd, brm, bE, bp, dT, drv, dpp);
+        make_prim_inv<S, double>(P, u, brd, brm, bE, bp, dT, 0.0, dpp, dir);
         if (S::RAIN) P.vr = dvr;
+        double F[S::D][S::NF];
+        flux_all<S>(P, F);
 #pragma unroll
-        for (int j = 0; j < S::D; ++j) {
-            double F[S::NF];
-            flux_dir<S, double>(P, j, F);
+        for (int j = 0; j < S::D; ++j)
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
-                s_fl[(j * S::NF + f) * STR + t] = F[f];
-                if (!DIFF && fx_field<S>(f)) ex[f] = max(ex[f], fx_expo(F[f]) + A.ref.q_vol[j]);
+                s_fl[(j * S::NF + f) * STR + t] = F[j][f];
+                if (!DIFF && fx_field<S>(f)) ex[f] = max(ex[f], fx_expo(F[j][f]) + A.ref.q_vol[j]);
             }
-        }
     }
 
     // ---- phase 1b (diffusion): F_j -= alpha du/dx_j at the node, so that the
