@@ -349,6 +349,21 @@ int upload_and_prepare(dg_ctx *c, const void *host) {
     return DG_OK;
 }
 
+// Whether a stage runs as face pass + stage kernel; else the stage kernel
+// evaluates the faces itself (both sides of each), one launch instead of two.
+// The results are the same bits.  Small meshes under DG_FACES_AUTO go inline:
+// up to the lines below, the second launch and its latency cost more than the
+// doubled face work (us per step, inline against face pass; float64 2-D: 100
+// tiles 59 / 75, 160 tiles 132 / 108; 3-D: 96 tiles 126 / 116; FP32-bulk: 128
+// tiles 44 / 54, 512 tiles 58 / 74, 800 tiles 74 / 77, 1024 tiles 89 / 87).
+// The members of an ensemble share the chip, so their total work counts.
+bool use_face_pass(const dg_ctx *c) {
+    if (!c->face_pass) return false;
+    if (c->cfg.faces != DG_FACES_AUTO || c->diff || c->in_ensemble) return true;
+    const long long tiles = (c->ne + c->epb - 1) / c->epb;
+    return tiles > (c->fp32 ? 4 * kSMs : (c->cfg.dim == 2 ? 2 * kSMs / 3 : 0));
+}
+
 // last: the stage that ends a time step (the sponge layer acts there);
 // fall_w: the stage's weight b_s dt in the step for the rain fall-out (0: the
 // stage adds nothing to it)
@@ -378,18 +393,19 @@ int do_stage(dg_ctx *c, const Launchers<Real> *L, const RefData<Real> &ref, int 
         if (st != DG_OK) return st;
     }
     if (c->column) return cuda_status(L->column(A, mode, c->stream));
-    if (c->face_pass) {
+    const bool pf = use_face_pass(c);
+    if (pf) {
         const int st = cuda_status(L->face(A, c->diff, c->stream));
         if (st != DG_OK) return st;
     }
-    if (!chunk_ev) return cuda_status(L->stage(A, mode, c->face_pass, c->diff, c->stream));
+    if (!chunk_ev) return cuda_status(L->stage(A, mode, pf, c->diff, c->stream));
     for (int k = 0; k < kChunks; ++k) {
         long long t0, t1;
         chunk_tiles(c, k, t0, t1);
         if (t1 > t0) {
             A.tile0 = (int)t0;
             A.ntiles = (int)(t1 - t0);
-            const int st = cuda_status(L->stage(A, mode, c->face_pass, c->diff, c->stream));
+            const int st = cuda_status(L->stage(A, mode, pf, c->diff, c->stream));
             if (st != DG_OK) return st;
         }
         if (cudaEventRecord(chunk_ev[k], c->stream) != cudaSuccess) return DG_ECUDA;
@@ -793,7 +809,7 @@ int dg_get_info(const dg_ctx *c, dg_info *info) {
     info->n_dofs = c->nodes * c->nf;
     info->state_bytes = (size_t)c->nodes * c->nf * c->rsz;
     info->device_bytes = c->device_bytes;
-    info->launches_per_stage = c->face_pass ? 2 : 1;   // column march and inline faces: 1
+    info->launches_per_stage = use_face_pass(c) ? 2 : 1;   // column march and inline faces: 1
     return DG_OK;
 }
 

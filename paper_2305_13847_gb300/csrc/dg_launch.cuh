@@ -36,6 +36,33 @@ inline int grid_for(size_t n, int threads) {
     return (int)(b > 0 ? b : 1);
 }
 
+// Launch, with programmatic dependent launch (dependents_go / dependents_wait,
+// dg_device.cuh) where it pays: the launch and the kernel's set-up overlap the
+// end of the kernel before it.  Blocks that start early sit where there is
+// room, not where they would be spread, so a grid of about one to six blocks
+// per SM ends up unbalanced (64x32 order 3 float64: 116 -> 178 us per step, the
+// same for a small grid behind a larger one).  It pays for a full chip of
+// threads and more (128x64 order 4 FP32-bulk: 99 -> 87 us per step) and in a
+// chain of kernels of at most one block per SM (`chain`; 20x10 order 3: 58 ->
+// 54 us).
+constexpr int kSMs = 152;
+
+template <class K, class... P>
+inline cudaError_t launch(K kern, int grid, int block, size_t smem, cudaStream_t st, bool chain,
+                          const P &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = ((chain && grid <= kSMs) || (long long)grid * block >= kSMs * 768) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <class S, typename Real>
 struct Impl {
     static constexpr bool F64 = std::is_same<Real, double>::value;
@@ -71,8 +98,7 @@ struct Impl {
             if (err != cudaSuccess) return err;
             attr = true;
         }
-        kern<<<A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st>>>(A);
-        return cudaGetLastError();
+        return launch(kern, A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st, true, A);
     }
 
     static cudaError_t prepare(const KArgs<Real> &A, bool diff, cudaStream_t st) {
@@ -102,8 +128,7 @@ struct Impl {
             if (err != cudaSuccess) return err;
             attr = true;
         }
-        kern<<<A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st>>>(A);
-        return cudaGetLastError();
+        return launch(kern, A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st, !PF, A);
     }
 
     static cudaError_t stage(const KArgs<Real> &A, int mode, bool pf, bool diff, cudaStream_t st) {
@@ -121,18 +146,14 @@ struct Impl {
 
     static cudaError_t face(const KArgs<Real> &A, bool diff, cudaStream_t st) {
         const int nb = A.M.fblk[0] + A.M.fblk[1] + A.M.fblk[2];
-        if (diff)
-            k_face<S, Real, true><<<nb, kFaceThreads, 0, st>>>(A);
-        else
-            k_face<S, Real, false><<<nb, kFaceThreads, 0, st>>>(A);
-        return cudaGetLastError();
+        return launch(diff ? &k_face<S, Real, true> : &k_face<S, Real, false>, nb, kFaceThreads, 0, st,
+                      false, A);
     }
 
     static cudaError_t alpha_vertex(const KArgs<Real> &A, cudaStream_t st) {
         const size_t nvt = (size_t)A.M.nv[0] * A.M.nv[1] * (S::D == 3 ? A.M.nv[2] : 1);
-        k_alpha_vertex<S::D, Real><<<grid_for(nvt, 256), 256, 0, st>>>(A.M, A.alphaK,
-                                                                        const_cast<Real *>(A.alphaV));
-        return cudaGetLastError();
+        return launch(&k_alpha_vertex<S::D, Real>, grid_for(nvt, 256), 256, 0, st, false, A.M,
+                      (const Real *)A.alphaK, const_cast<Real *>(A.alphaV));
     }
 
     static cudaError_t split(const KArgs<Real> &A, double *T, double *rv, double *rc, double *pp,
@@ -208,15 +229,25 @@ RefData<double> scaled_ref64(int order, const double two_over_h[3]);
 
 }  // namespace dgm
 
+namespace dgm {
+// Tile of the kernels of one storage type: 128 threads, but 256 for float32 in
+// 2-D (128 threads cost the 256-member ensemble 3 %).  Float64 in 2-D: 128
+// threads spread small meshes over more SMs (20x10 order 3: 75 us per step
+// against 84) and waste fewer lanes (order 4: 125 of 128; 128x64 with rain,
+// four steps: 1.52 ms against 1.62 at 256 and 1.75 at 64).
+template <int D, int K, bool RAIN, typename Real>
+using TileShape = Shape<D, K, RAIN, (D == 2 && sizeof(Real) == sizeof(float)) ? 256 : 128>;
+}  // namespace dgm
+
 #define DGM_DEFINE_LAUNCHERS(NAME, DIM, REAL)                                          \
     namespace dgm {                                                                    \
     const Launchers<REAL> *NAME(int K, int rain) {                                     \
         static const Launchers<REAL> t[5][2] = {                                       \
-            {Impl<Shape<DIM, 1, false>, REAL>::table(), Impl<Shape<DIM, 1, true>, REAL>::table()}, \
-            {Impl<Shape<DIM, 2, false>, REAL>::table(), Impl<Shape<DIM, 2, true>, REAL>::table()}, \
-            {Impl<Shape<DIM, 3, false>, REAL>::table(), Impl<Shape<DIM, 3, true>, REAL>::table()}, \
-            {Impl<Shape<DIM, 4, false>, REAL>::table(), Impl<Shape<DIM, 4, true>, REAL>::table()}, \
-            {Impl<Shape<DIM, 5, false>, REAL>::table(), Impl<Shape<DIM, 5, true>, REAL>::table()}, \
+            {Impl<TileShape<DIM, 1, false, REAL>, REAL>::table(), Impl<TileShape<DIM, 1, true, REAL>, REAL>::table()}, \
+            {Impl<TileShape<DIM, 2, false, REAL>, REAL>::table(), Impl<TileShape<DIM, 2, true, REAL>, REAL>::table()}, \
+            {Impl<TileShape<DIM, 3, false, REAL>, REAL>::table(), Impl<TileShape<DIM, 3, true, REAL>, REAL>::table()}, \
+            {Impl<TileShape<DIM, 4, false, REAL>, REAL>::table(), Impl<TileShape<DIM, 4, true, REAL>, REAL>::table()}, \
+            {Impl<TileShape<DIM, 5, false, REAL>, REAL>::table(), Impl<TileShape<DIM, 5, true, REAL>, REAL>::table()}, \
         };                                                                             \
         if (K < 1 || K > 5) return nullptr;                                            \
         return &t[K - 1][rain ? 1 : 0];                                                \

@@ -241,16 +241,15 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
     const int e = bidx * S::EPB + el;
     const bool valid = t < STR && e < A.M.ne;
     double v[S::NTR];
+    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
+    if (t < FxExp<S, DIFF>::N) s_e[t] = 0;
+    if (DIFF && t < 2 * S::EPB) s_red[t] = 0.0;
+    dependents_wait();
+    __syncthreads();
     if (valid) {
         const size_t nodes = (size_t)A.M.ne * S::NP, gi = (size_t)e * S::NP + a;
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) v[f] = A.Uin[f * nodes + gi];
-    }
-    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
-    if (t < FxExp<S, DIFF>::N) s_e[t] = 0;
-    if (DIFF && t < 2 * S::EPB) s_red[t] = 0.0;
-    __syncthreads();
-    if (valid) {
         double vr;
         derive_and_store<S, double>(A, v, e, a, vert_index<S::D>(A.M, e), -1.0, v[S::NF], v[S::NF + 1],
                                     v[S::NF + 2], vr);
@@ -321,6 +320,9 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     const bool valid = (t < STR) && (e < ne);
     const size_t gi = (size_t)e * S::NP + a;
 
+    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
+    if (t < X::N) s_e[t] = 0;
+    dependents_wait();
     // the node's state and derived fields: loads issued first, so that their
     // latency overlaps the set-up below
     double u[S::NF], dT = 0.0, dir = 1.0, dpp = 0.0, dgm = 0.0, dvr = 0.0;
@@ -338,8 +340,6 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     // face pass: copy the tile's face values to shared memory while the
     // nodal phase runs (one contiguous block per face)
     if (PF) cp_async_faces<S, double, NFP>(A.fbuf, A.ftab, s_fh, bidx, min(S::EPB, ne - bidx * S::EPB));
-    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
-    if (t < X::N) s_e[t] = 0;
     if (DIFF || !PF) {
         if (t < S::EPB && bidx * S::EPB + t < ne) {
             int im[3];
@@ -489,7 +489,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     if (!bad) {
         // in place: each thread converts the words that it wrote or scanned
         if (valid) {
-#pragma unroll
+#pragma unroll 1
             for (int j = 0; j < S::D; ++j)
 #pragma unroll
                 for (int f = 0; f < S::NF; ++f) {
@@ -516,7 +516,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
             double rr = 0.0;      // rain density
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) a2[f] = a1[f] = 0;
-#pragma unroll
+#pragma unroll 1
             for (int j = 0; j < S::D; ++j) {
                 const int aj = digit<S::D, S::P1>(a, j);
                 const int st = stride_of<S::P1>(j);
@@ -626,6 +626,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
 template <class S, bool DIFF>
 __global__ void __launch_bounds__(S::NT) k_prepare64(KArgs<double> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dependents_go();
     prepare_block64<S, DIFF>(A, blockIdx.x + A.tile0, smem_raw);
 }
 
@@ -642,6 +643,7 @@ constexpr int stage64_min_blocks() {
 template <class S, int MODE, bool PF, bool DIFF>
 __global__ void __launch_bounds__(S::NT, (stage64_min_blocks<S, DIFF>())) k_stage64(KArgs<double> A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    dependents_go();
     stage_block64<S, MODE, PF, DIFF>(A, blockIdx.x + A.tile0, smem_raw);
 }
 
