@@ -348,7 +348,7 @@ __device__ __forceinline__ double rho_vs(double T, double invT) {
 __device__ __forceinline__ float rho_vs_f32(float T) {
     const float l2e = 1.4426950408889634f;
     return (float)kRvs0 * exp2f((float)(kEsA - 1.0) * __log2f(T * (float)kInvTref) +
-                                (float)kEsB * l2e * ((float)kInvTref - __frcp_rn(T)));
+                                (float)kEsB * l2e * ((float)kInvTref - frcp(T)));
 }
 
 // float64 rho_vs(T) and d rho_vs / dT from the Taylor table (dg_math.cuh).
@@ -453,7 +453,7 @@ __device__ __forceinline__ SplitResult split_point(double rd, double rm, double 
     const double X = fma(-rm, kLprime, re);
     const float rmf = narrow(rm);
     const float cuf = (float)kCvd * narrow(rd) + (float)kCvv * rmf + (float)kCl * narrow(rr);
-    const float tuf = fmaf(narrow(X), __frcp_rn(cuf), (float)kTref);
+    const float tuf = fmaf(narrow(X), frcp(cuf), (float)kTref);
     const float rvs32 = rho_vs_f32(tuf);
     bool sat;
     double rvs_u = 0.0, tu = 0.0;
@@ -484,12 +484,12 @@ __device__ __forceinline__ SplitResult split_point(double rd, double rm, double 
         const int n32 = cap < 30 ? cap : 30;
         for (int it = 0; it < n32; ++it) {
             const float rvs = rho_vs_f32(t);
-            const float it_ = __frcp_rn(t);
+            const float it_ = frcp(t);
             const float drvs = rvs * it_ * (am1 + bb * it_);
             const float heat = cdf + clv * rvs;
             const float h = heat * (t - tref) + rvs * lp - ref;
             const float dh = heat + (clv * (t - tref) + lp) * drvs;
-            const float dt = h * __frcp_rn(dh);
+            const float dt = h * frcp(dh);
             t -= dt;
             if (fabsf(dt) <= 2e-6f * t) break;
         }
@@ -511,14 +511,14 @@ __device__ __forceinline__ SplitResult split_point(double rd, double rm, double 
         // float64 residual H + H' d0, together within 2^-44 of d (|d| <= 3e-4 K,
         // so 2e-17 K); two float64 operations instead of a reciprocal's and a
         // product's four
-        const float ridh = __frcp_rn(narrow(dh));
+        const float ridh = frcp(narrow(dh));
         const float df = -narrow(h) * ridh;
         if (fabsf(df) <= 3e-4f) {
             const double d0 = widen(df);
             const float d1 = -narrow(fma(dh, d0, h)) * ridh;
             // H'' = 2 (c_vv - c_l) rho_vs' + (c_vv - c_l)(T - T_ref) + L') rho_vs'',
             // rho_vs'' = rho_vs (phi1^2 + phi1'), phi1' = -(a-1)/T^2 - 2b/T^3
-            const float itf = __frcp_rn(tf ? t : narrow(t0)), rvf = narrow(rvs);
+            const float itf = frcp(tf ? t : narrow(t0)), rvf = narrow(rvs);
             const float p1f = itf * (am1 + bb * itf);               // (ln rho_vs)
             const float d2rvs = rvf * (p1f * p1f - itf * itf * (am1 + 2.0f * bb * itf));
             const float d2h = 2.0f * clv * (rvf * p1f) + narrow(lat) * d2rvs;
@@ -575,7 +575,7 @@ __device__ __forceinline__ float rain_velocity(float rr, float rm, const MeshDat
     const float rrp = rr > 0.0f ? rr : 0.0f;
     const float rw = M.rho_w_f > 0.0f ? M.rho_w_f : rm + rr;
     if (!(rrp > 0.0f) || !(rw > 0.0f)) return 0.0f;
-    return M.kvr_f * exp2f(0.125f * __log2f(rrp * __frcp_rn(rw)));
+    return M.kvr_f * exp2f(0.125f * __log2f(rrp * frcp(rw)));
 }
 
 // Per-node split plus the node-local quantities the next operator needs.
@@ -665,14 +665,14 @@ __device__ __forceinline__ NodeDerived node_derived_bulk(const float *u, int im,
     const double rd = brd + widen(u[0]);
     const double rm = brm + widen(u[1]);
     const double rr = RAIN ? widen(u[2]) : 0.0;
-    const double re = (bE + widen(u[ie])) - widen(0.5f * msq * __frcp_rn(rhof));
+    const double re = (bE + widen(u[ie])) - widen(0.5f * msq * frcp(rhof));
     // T_u = T_ref + X / C_u, X = E_int - rho_m L'.  The float32 T_u (from the
     // float32 X, within ~1e-5 K) decides saturation and starts the pre-solve;
     // X and T_u in float64 are formed only where T = T_u (unsaturated) or the
     // decision is close
     const float ref = narrow(re);
     const float cuf = (float)kCvd * rdf + (float)kCvv * rmf + (float)kCl * rrf;
-    const float rcu = __frcp_rn(cuf);
+    const float rcu = frcp(cuf);
     const float tuf = fmaf(fmaf(-rmf, (float)kLprime, ref), rcu, (float)kTref);
     const float rvs32 = rho_vs_f32(tuf);
     bool sat;
@@ -709,11 +709,11 @@ __device__ __forceinline__ NodeDerived node_derived_bulk(const float *u, int im,
         const int n32 = M.newton_cap < 40 ? M.newton_cap : 40;
         for (int it = 0; it < n32; ++it) {
             const float rvs = rho_vs_f32(t);
-            const float drvs = drho_vs_f32(rvs, __frcp_rn(t));
+            const float drvs = drho_vs_f32(rvs, frcp(t));
             const float heat = cdf + clv * rvs;
             const float h = heat * (t - tref) + rvs * lp - ref;
             const float dh = heat + (clv * (t - tref) + lp) * drvs;
-            const float dt = h * __frcp_rn(dh);
+            const float dt = h * frcp(dh);
             t -= dt;
             // a step of at most 2e-3 K leaves at most (H''/2H') dt^2 < 2e-7 K;
             // the float64 correction below takes the rest
@@ -732,9 +732,9 @@ __device__ __forceinline__ NodeDerived node_derived_bulk(const float *u, int im,
         const double cdry = fma(kCvd, rd, kCl * (rm + rr));
         const double h = fma(fma(kCvv - kCl, rvs, cdry), T32 - kTref, fma(rvs, kLprime, -re));
         const float rvsf = narrow(rvs);
-        const float drvs = drho_vs_f32(rvsf, __frcp_rn(t));
+        const float drvs = drho_vs_f32(rvsf, frcp(t));
         const float dh = cdf + clv * rvsf + (clv * (t - tref) + lp) * drvs;
-        const float dT = narrow(h) / dh;
+        const float dT = narrow(h) * frcp(dh);
         o.T = T32 - widen(dT);
         o.rv = rvs - widen(drvs * dT);
         Tf = narrow(o.T);
@@ -792,7 +792,7 @@ constexpr int kBsN = 12;  // 0 T_bar, 1 rho_v_bar, 2 R_bar = rho_vs(T_bar), 3 rh
 // iTb = 1/T_bar and bTb = b/T_bar from the table, iT = 1/T (no divisions)
 __device__ __forceinline__ float phi_of(float tau, float iTb, float bTb, float iT) {
     const float am1 = (float)(kEsA - 1.0);
-    return am1 * log1pf(tau * iTb) + bTb * (tau * iT);
+    return am1 * log1p_small(tau * iTb) + bTb * (tau * iT);
 }
 
 template <bool RAIN>
@@ -810,14 +810,14 @@ __device__ __forceinline__ NodeDerived node_derived_pert(const float *u, int im,
     float msq = 0.0f;
     for (int j = 0; j < d; ++j) msq = fmaf(u[im + j], u[im + j], msq);
     // rho e - (base identity) = E' - |m|^2/(2 rho) + energy residual
-    const float de = (u[ie] - 0.5f * msq * __frcp_rn(rho)) + eres;
+    const float de = (u[ie] - 0.5f * msq * frcp(rho)) + eres;
     const float c0 = cvd * rdp + cl * (rmp + rrp);            // C - C_bar without the nu part
     // unsaturated candidate: rho_v = rho_m, nu_u = rho_m' + (rho_m_bar - rho_v_bar)
     const float nu_u = rmp + cqb;
     const float Cu = Cb + c0 + (cvv - cl) * nu_u;
-    const float tau_u = (de - (c0 + (cvv - cl) * nu_u) * dTb - nu_u * lp) * __frcp_rn(Cu);
+    const float tau_u = (de - (c0 + (cvv - cl) * nu_u) * dTb - nu_u * lp) * frcp(Cu);
     // saturated iff rho_m > rho_vs(T_u) <=> rho_m' + Q_bar - R_bar expm1(phi(tau_u)) > 0
-    const float em_u = expm1f(phi_of(tau_u, iTb, bTb, __frcp_rn(Tb + tau_u)));
+    const float em_u = expm1_small(phi_of(tau_u, iTb, bTb, frcp(Tb + tau_u)));
     const bool sat = rmp + Qb - Rb * em_u > 0.0f;
     float tau, nu, deficit = 0.0f;
     bool conv = true;
@@ -841,15 +841,15 @@ __device__ __forceinline__ NodeDerived node_derived_pert(const float *u, int im,
         const int n32 = M.newton_cap < 40 ? M.newton_cap : 40;
         for (int it = 0; it < n32; ++it) {
             const float T = Tb + tau;
-            const float iT = __frcp_rn(T);
-            const float em = expm1f(phi_of(tau, iTb, bTb, iT));
+            const float iT = frcp(T);
+            const float em = expm1_small(phi_of(tau, iTb, bTb, iT));
             const float nus = Db + Rb * em;                     // rho_vs(T) - rho_v_bar
             const float p1 = iT * (am1 + bb * iT);              // d phi / d tau
             const float dnu = Rb * (1.0f + em) * p1;
             const float C = Cb + c0 + (cvv - cl) * nus;
             const float h = C * tau + (c0 + (cvv - cl) * nus) * dTb + nus * lp - de;
             const float dh = C + ((cvv - cl) * (tau + dTb) + lp) * dnu;
-            const float step = h * __frcp_rn(dh);
+            const float step = h * frcp(dh);
             tau -= step;
             // done once the step s is at most 2e-3 K: Newton leaves an error
             // of at most (H''/2H') s^2, and H''/2H' < 0.05 /K on the saturated
@@ -870,7 +870,7 @@ __device__ __forceinline__ NodeDerived node_derived_pert(const float *u, int im,
             }
             prev = as;
         }
-        if (!have_nu) nu = Db + Rb * expm1f(phi_of(tau, iTb, bTb, __frcp_rn(Tb + tau)));
+        if (!have_nu) nu = Db + Rb * expm1_small(phi_of(tau, iTb, bTb, frcp(Tb + tau)));
     }
     const float T = Tb + tau;
     o.Tf = T;
