@@ -82,12 +82,12 @@ struct AdjArgs {
     RefData<double> ref;
     const double *U;        // state (ABI layout)
     const double *derived;  // T, rho_v, p' (, G, v_r) of U
-    const double *trace;    // traces of U, [2D][NTR][ne][NFP1]
+    const double *trace;    // traces of U (TraceLayout)
     const double *bnode, *bface;  // base tables
     const double *rvs_tab;  // rho_vs Taylor table (dg_math.cuh)
     const double *w;        // adjoint input (ABI layout)
     double *ubar_part;      // [NTR][nodes]: adjoints of U (NF) and of T, rho_v, p'
-    double *tadj;           // [2D][NTR][ne][NFP1]: neighbour trace adjoints
+    double *tadj;           // neighbour trace adjoints, as the traces
     double *out;            // [NF][nodes]
     double alpha, beta, gamma;
 };
@@ -300,19 +300,18 @@ __device__ __forceinline__ void face_vjp(const AdjArgs &A, const double *s_w, do
                                          int face, int q, int e2) {
     constexpr int STR = S::EPB * S::NP;
     const MeshData &M = A.M;
-    const int ne = M.ne;
     const int s = (face & 1) ? 1 : -1;
     double tm[S::NTR], tp[S::NTR];
 #pragma unroll
     for (int fld = 0; fld < S::NTR; ++fld)
-        tm[fld] = has_trace<S>(fld, J) ? A.trace[(((size_t)face * S::NTR + fld) * ne + e2) * S::NFP1 + q]
+        tm[fld] = has_trace<S>(fld, J) ? A.trace[TraceLayout<S, double>::face(e2, face) + fld * S::NFP1 + q]
                                        : 0.0;
     const int nb = neighbour<S::D>(M, e2, J, s);
     if (nb >= 0) {
         const int fo = 2 * J + (s > 0 ? 0 : 1);
 #pragma unroll
         for (int fld = 0; fld < S::NTR; ++fld)
-            tp[fld] = has_trace<S>(fld, J) ? A.trace[(((size_t)fo * S::NTR + fld) * ne + nb) * S::NFP1 + q]
+            tp[fld] = has_trace<S>(fld, J) ? A.trace[TraceLayout<S, double>::face(nb, fo) + fld * S::NFP1 + q]
                                            : 0.0;
     } else {
 #pragma unroll
@@ -395,7 +394,7 @@ __device__ __forceinline__ void face_vjp(const AdjArgs &A, const double *s_w, do
         const int fo = 2 * J + (s > 0 ? 0 : 1);
 #pragma unroll
         for (int fld = 0; fld < S::NTR; ++fld)
-            A.tadj[(((size_t)fo * S::NTR + fld) * ne + nb) * S::NFP1 + q] = tpb[fld];
+            A.tadj[TraceLayout<S, double>::face(nb, fo) + fld * S::NFP1 + q] = tpb[fld];
     } else {
         // wall ghost: tp = tm with m_J negated
 #pragma unroll
@@ -583,7 +582,7 @@ __global__ void k_adj_gather(AdjArgs A) {
                 const double c = sd ? A.ref.lp[aj] : A.ref.lm[aj];
 #pragma unroll
                 for (int fld = 0; fld < S::NTR; ++fld)
-                    xb[fld] += c * A.tadj[(((size_t)face * S::NTR + fld) * ne + e) * S::NFP1 + q];
+                    xb[fld] += c * A.tadj[TraceLayout<S, double>::face(e, face) + fld * S::NFP1 + q];
             }
         }
         double u[S::NF];

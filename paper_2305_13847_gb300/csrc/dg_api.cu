@@ -453,9 +453,10 @@ void mesh_float_copies(MeshData &M) {
     M.alpha_pre_f = (float)M.alpha_pre;
 }
 
-// face grid of the face pass; returns the length (in elements) of its
-// face-major buffer [faces normal to e_0 | e_1 | e_2][per_point][NFP1]
-long long set_face_layout(dg_ctx *c, int per_point) {
+// face grid of the face pass; returns the bytes of its face-major buffer
+// [faces normal to e_0 | e_1 | e_2], per_point fields per face point in
+// blocks of whole 16-byte pieces (FaceLayout)
+size_t set_face_layout(dg_ctx *c, int per_point) {
     MeshData &M = c->M;
     const dg_config &g = c->cfg;
     for (int j = 0; j < 3; ++j) {
@@ -469,7 +470,8 @@ long long set_face_layout(dg_ctx *c, int per_point) {
         M.nfaces[j] = (int)nfj;
         M.fblk[j] = (int)((nfj * c->nfp1 + kFaceThreads - 1) / kFaceThreads);
     }
-    return ((long long)M.nfaces[0] + M.nfaces[1] + M.nfaces[2]) * per_point * c->nfp1;
+    const size_t face = ((size_t)per_point * c->nfp1 * c->rsz + 15) / 16 * 16;
+    return ((size_t)M.nfaces[0] + M.nfaces[1] + M.nfaces[2]) * face;
 }
 
 // index in the face-major face buffer of every element's 2D faces, [ne][2D]
@@ -543,7 +545,7 @@ int upload_base(dg_ctx *c, const double *node_tab, const double *face_tab) {
 int ensure_adjoint(dg_ctx *c) {
     if (c->ubar_part) return DG_OK;
     const size_t state = (size_t)c->nodes * c->nf * sizeof(double);
-    const size_t trace = (size_t)2 * c->cfg.dim * c->ntr * c->ne * c->nfp1 * sizeof(double);
+    const size_t trace = (size_t)2 * c->cfg.dim * c->ne * c->trace_face * sizeof(double);
     int st = DG_OK;
     for (int i = 0; i < 3 && st == DG_OK; ++i) st = alloc(c, &c->adjX[i], state);
     for (int i = 0; i < 3 && st == DG_OK; ++i) st = alloc(c, (void **)&c->adjL[i], state);
@@ -653,6 +655,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
         c->L32 = g.dim == 2 ? launchers_d2_f32(g.order, g.rain) : launchers_d3_f32(g.order, g.rain);
         c->nf = c->L32->nf; c->np = c->L32->np; c->nfp1 = c->L32->nfp1;
         c->nd = c->L32->nd; c->ntr = c->L32->ntr; c->epb = c->L32->epb;
+        c->trace_face = c->L32->trace_face;
     } else {
         // DG_FP64_FFC is float64 too: its contractions run on the integer pipe
         // with more bits than the float32 pairs of that form had
@@ -660,6 +663,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
         c->LA = g.dim == 2 ? adj_launchers_d2(g.order, g.rain) : adj_launchers_d3(g.order, g.rain);
         c->nf = c->L64->nf; c->np = c->L64->np; c->nfp1 = c->L64->nfp1;
         c->nd = c->L64->nd; c->ntr = c->L64->ntr; c->epb = c->L64->epb;
+        c->trace_face = c->L64->trace_face;
     }
     c->ne = ne;
     c->nodes = ne * np;
@@ -692,7 +696,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
     // (measured: float64 -21 %, float32 forms -8 to -11 % per step)
     c->face_pass = g.faces == DG_FACES_AUTO || g.faces == DG_FACES_PASS;
     c->column = g.faces == DG_FACES_COLUMN;
-    const long long fbuf_len = set_face_layout(c, nf);
+    c->fbuf_bytes = set_face_layout(c, nf);
     mesh_float_copies(M);
     // the volume derivative and lift tables pre-scaled by 2/h_j of this
     // mesh, float64 and their float32 roundings
@@ -718,7 +722,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
 
     DeviceGuard dg(c->device);
     const size_t state = (size_t)c->nodes * nf * c->rsz;
-    const size_t trace = (size_t)2 * g.dim * c->ntr * ne * c->nfp1 * c->rsz;
+    const size_t trace = (size_t)2 * g.dim * ne * c->trace_face * c->rsz;
     c->nred = std::min<long long>(kGridStrideBlocks, (c->nodes + kRedThreads - 1) / kRedThreads);
     int st = DG_OK;
     if (st == DG_OK) st = alloc(c, &c->U[0], state);
@@ -740,7 +744,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
     if (st == DG_OK) st = alloc(c, (void **)&c->rvs_tab, sizeof(double) * kTabStride * kTabN);
     if (st == DG_OK && M.pert_split)
         st = alloc(c, (void **)&c->bsplit, sizeof(float) * kBsN * M.nzlev_node);
-    if (st == DG_OK && c->face_pass) st = alloc(c, &c->fbuf, (size_t)fbuf_len * c->rsz);
+    if (st == DG_OK && c->face_pass) st = alloc(c, &c->fbuf, c->fbuf_bytes);
     if (st == DG_OK && c->face_pass) {
         const std::vector<int> tab = face_table(c);
         st = alloc(c, (void **)&c->ftab, sizeof(int) * tab.size());
@@ -1196,13 +1200,14 @@ int dg_set_stabilisation(dg_ctx *c, const dg_stabilisation *sp) {
         if (st == DG_OK) st = alloc(c, &c->dtrace[0], dtr);
         if (st == DG_OK) st = alloc(c, &c->dtrace[1], dtr);
         if (st == DG_OK) {
-            const long long len = set_face_layout(c, 2 * c->nf);
+            const size_t bytes = set_face_layout(c, 2 * c->nf);
             void *nb = nullptr;
-            st = alloc(c, &nb, (size_t)len * c->rsz);
+            st = alloc(c, &nb, bytes);
             if (st == DG_OK) {
                 cudaFree(c->fbuf);
-                c->device_bytes -= (size_t)(len / 2) * c->rsz;
+                c->device_bytes -= c->fbuf_bytes;
                 c->fbuf = nb;
+                c->fbuf_bytes = bytes;
             } else {
                 set_face_layout(c, c->nf);
             }

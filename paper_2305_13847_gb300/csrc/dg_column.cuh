@@ -110,7 +110,6 @@ __device__ __forceinline__ void col_hface(const KArgs<Real> &A, const Real *s_tr
                                           int hi_y) {
     using C = ColShape<S>;
     const MeshData &M = A.M;
-    const int ne = M.ne;
     const int ncol = S::D == 3 ? M.n[0] * M.n[1] : M.n[0];
     const ColSide lo = col_side<S>(M, cx0, cy0, lo_x, lo_y);
     const ColSide hi = col_side<S>(M, cx0, cy0, hi_x, hi_y);
@@ -128,11 +127,7 @@ __device__ __forceinline__ void col_hface(const KArgs<Real> &A, const Real *s_tr
         } else if (sd.kind == 2) {
             const int e = sd.glob + ncol * iz;
             const int face = 2 * J + (side == 0 ? 1 : 0);
-#pragma unroll
-            for (int fld = 0; fld < S::NTR; ++fld)
-                tr[fld] = has_trace<S>(fld, J)
-                              ? A.trace_in[(((size_t)face * S::NTR + fld) * ne + e) * S::NFP1 + q]
-                              : Real(0);
+            load_traces<S, Real, J>(A.trace_in, e, face, q, tr);
         }
     }
     // slip wall: the ghost copies the other side with m.n mirrored
@@ -414,7 +409,8 @@ __global__ void __launch_bounds__(ColShape<S>::NT, ColShape<S>::MINB) k_column(K
 #pragma unroll
                 for (int fld = 0; fld < S::NTR; ++fld)
                     if (has_trace<S>(fld, j))
-                        A.trace_out[(((size_t)face * S::NTR + fld) * M.ne + e) * S::NFP1 + q] = tr[fld];
+                        A.trace_out[TraceLayout<S, Real>::face(e, face) +
+                                    TraceLayout<S, Real>::at(fld, q, S::NFP1)] = tr[fld];
             }
         }
         __syncthreads();

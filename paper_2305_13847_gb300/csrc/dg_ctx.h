@@ -17,7 +17,7 @@ struct dg_ctx {
     int fp32 = 0;
     const Launchers<double> *L64 = nullptr;
     const Launchers<float> *L32 = nullptr;
-    int nf = 0, np = 0, nfp1 = 0, nd = 0, ntr = 0, epb = 0;
+    int nf = 0, np = 0, nfp1 = 0, nd = 0, ntr = 0, epb = 0, trace_face = 0;
     long long ne = 0, nodes = 0;
     size_t rsz = 8;
     MeshData M;
@@ -37,6 +37,7 @@ struct dg_ctx {
     bool face_pass = false;      // faces in k_face (DG_FACES_PASS) instead of in the stage kernel
     bool column = false;         // DG_FACES_COLUMN: the column-march stage kernel (float32 forms)
     void *fbuf = nullptr;        // face pass: fluxes per face point
+    size_t fbuf_bytes = 0;
     int *ftab = nullptr;         // face pass: index in fbuf of each element's 2D faces [ne][2D]
     // artificial diffusion and sponge layer (dg_set_stabilisation)
     dg_stabilisation stab{};

@@ -141,20 +141,20 @@ struct KArgs {
     const Real *Un;        // U^n for the stage combination (may equal Uin)
     Real *Uout;            // MODE_RHS: dU/dt; MODE_STAGE: new stage state
     Real *derived;         // [ND][nodes]: T, rho_v (float64: 1/rho, see keep_rv), p' [, G_rm, v_r]
-    const Real *trace_in;  // traces of Uin:   [2D][NTR][ne][NFP1]
+    const Real *trace_in;  // traces of Uin (TraceLayout)
     Real *trace_out;       // traces of Uout (MODE_STAGE)
     const Real *bnode;     // base at node levels [4][nzlev_node]: rho_d, rho_m, E, p
     const Real *bface;     // base at face levels [4][nzlev_face]
     const double *bnode_d; // float64 copy for the split
     const double *rvs_tab; // rho_vs Taylor table: [kTabN][kTabStride] (dg_math.cuh)
     const float *bsplit;   // DG_FP32_PERT: split of the base state per node level [kBsN][nzlev_node]
-    Real *fbuf;            // face pass: G along +e_j of every face, face-major [faces][NFP][NFP1]
-                           // (faces normal to e_0, then e_1, e_2); with diffusion NFP = 2 NF:
+    Real *fbuf;            // face pass: G along +e_j of every face, face-major (FaceLayout;
+                           // faces normal to e_0, then e_1, e_2); with diffusion 2 NF fields:
                            // flux, then S = alpha [[u]] / 2
     const int *ftab;       // face pass: index in fbuf of each element's 2D faces [ne][2D]
     Real *alphaK;          // diffusion: [2][ne] alpha_u, alpha_r per element (of the state produced)
     const Real *alphaV;    // diffusion: [2][nv] continuous coefficient at the vertices
-    const Real *dtrace_in; // diffusion: d/dx_j traces of Uin  [2D][NF][ne][NFP1]
+    const Real *dtrace_in; // diffusion: d/dx_j traces of Uin  [ne][2D][NF][NFP1]
     Real *dtrace_out;      // diffusion: d/dx_j traces of Uout
     const Real *sponge;    // sponge delta_R at the node levels (last stage of a step) or null
     Real alpha, beta, gdt; // Uout = alpha Un + beta Uin + gdt dU/dt
@@ -249,6 +249,71 @@ __device__ __forceinline__ int face_q_vert(int j, int q) {
     if (D == 2) return q;           // j == 0: remaining direction is the vertical
     return q / P1;                  // j = 0 or 1: remaining (., vertical)
 }
+
+// Which trace fields a face carries: T enters the face flux only through the
+// rain's energy flux on faces normal to e_z, so the other faces hold no
+// temperature trace (its slot in the trace buffer is neither written nor read)
+template <class S>
+__host__ __device__ constexpr bool has_trace(int fld, int j) {
+    return fld != S::NF || j == S::VERT;
+}
+
+__host__ __device__ constexpr int round_up_to(int n, int m) { return (n + m - 1) / m * m; }
+
+// Trace buffer [ne][2D][FACE]: the values of one face of one element are
+// contiguous and every field's offset in them is a compile-time constant.
+// float64: [NTR][NFP1].  float32: the fields as interleaved pairs (64-bit
+// accesses, paired fmas), in the slot order U, rho_v, p', T, so that an odd
+// field out and the temperature stand in rows of their own at the end.
+template <class S, typename Real>
+struct TraceLayout {
+    static constexpr bool PAIRS = sizeof(Real) == sizeof(float);
+    static constexpr int NPAIR = PAIRS ? (S::NTR - 1) / 2 : 0;
+    static constexpr int FACE = PAIRS ? round_up_to(S::NTR * S::NFP1, 4) : S::NTR * S::NFP1;
+    __host__ __device__ static constexpr int slot(int fld) {
+        return !PAIRS || fld < S::NF ? fld : (fld == S::NF ? S::NF + 2 : fld - 1);
+    }
+    __host__ __device__ static constexpr int field(int sl) {
+        return !PAIRS || sl < S::NF ? sl : (sl == S::NF + 2 ? S::NF : sl + 1);
+    }
+    // offset of field fld at item t of rows of n items
+    __host__ __device__ static constexpr int at(int fld, int t, int n) {
+        return slot(fld) < 2 * NPAIR ? ((slot(fld) >> 1) * n + t) * 2 + (slot(fld) & 1) : slot(fld) * n + t;
+    }
+    __host__ __device__ static constexpr size_t face(int e, int f) { return ((size_t)e * S::NFACE + f) * FACE; }
+};
+
+// the traces of face (e, f) normal to e_J at point q
+template <class S, typename Real, int J>
+__device__ __forceinline__ void load_traces(const Real *buf, int e, int f, int q, Real *t) {
+    using L = TraceLayout<S, Real>;
+    const Real *b = buf + L::face(e, f);
+    if constexpr (L::PAIRS) {
+        const float2 *b2 = reinterpret_cast<const float2 *>(b) + q;
+#pragma unroll
+        for (int p = 0; p < L::NPAIR; ++p) {
+            const float2 v = b2[p * S::NFP1];
+            t[L::field(2 * p)] = v.x;
+            t[L::field(2 * p + 1)] = v.y;
+        }
+    }
+#pragma unroll
+    for (int sl = 2 * L::NPAIR; sl < S::NTR; ++sl)
+        t[L::field(sl)] = has_trace<S>(L::field(sl), J) ? b[sl * S::NFP1 + q] : Real(0);
+}
+
+// Face values [faces][FACE] of the face pass (N fields, N = NF or with
+// diffusion 2 NF), and a tile's in shared memory: a whole number of 16-byte
+// pieces per face for the asynchronous copy.  float64: [N][NFP1]; float32:
+// field pairs, then an odd field's row.
+template <class S, typename Real, int N>
+struct FaceLayout {
+    static constexpr int NPAIR = sizeof(Real) == sizeof(float) ? N / 2 : 0;
+    static constexpr int FACE = round_up_to(N * S::NFP1 * (int)sizeof(Real), 16) / (int)sizeof(Real);
+    __host__ __device__ static constexpr int at(int fld, int q) {
+        return fld < 2 * NPAIR ? ((fld >> 1) * S::NFP1 + q) * 2 + (fld & 1) : fld * S::NFP1 + q;
+    }
+};
 
 // Nodal fluxes of a float32 tile: interleaved field pairs (2p, 2p + 1), the
 // last pair padded when n_f is odd, [D][(n_f + 1) / 2][STR][2], so that the
@@ -1011,21 +1076,14 @@ __device__ __forceinline__ Real wave_speed(const Prim<S::D, S::RAIN, Real> &P) {
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 
-// trace of a nodal field on face (j, s) at face point q: sum_i l_i(s) v(line node i)
-template <class S, typename Real>
+// trace of a nodal field on face (j, s) at face point q: sum_i l_i(s) v(line
+// node i), the nodes STEP apart
+template <class S, typename Real, int STEP = 1>
 __device__ __forceinline__ Real interp_face(const Real *v, const Real *ls, int j, int q) {
     Real acc = Real(0);
 #pragma unroll
-    for (int i = 0; i < S::P1; ++i) acc = fma(ls[i], v[line_node<S::D, S::P1>(j, q, i)], acc);
+    for (int i = 0; i < S::P1; ++i) acc = fma(ls[i], v[STEP * line_node<S::D, S::P1>(j, q, i)], acc);
     return acc;
-}
-
-// Which trace fields a face carries: T enters the face flux only through the
-// rain's energy flux on faces normal to e_z, so the other faces hold no
-// temperature trace (its slot in the trace buffer is neither written nor read)
-template <class S>
-__host__ __device__ constexpr bool has_trace(int fld, int j) {
-    return fld != S::NF || j == S::VERT;
 }
 
 // Programmatic dependent launch: the next kernel of the stream may start its
@@ -1044,40 +1102,55 @@ __device__ __forceinline__ void dependents_wait() { asm volatile("griddepcontrol
 // ends (same fma chain as interp_face).  DIFF: also the traces of
 // d/dx_J U, (2/h_J) sum_i l_i'(+-1) U(line node i), for the interior-penalty
 // terms.
-template <class S, typename Real, bool DIFF, int J>
-__device__ __forceinline__ void write_line(const KArgs<Real> &A, const RefData<Real> &ref,
-                                           const Real *s_tr, Real *trace_out, int el, int e, int q) {
+template <class S, bool DIFF, int J>
+__device__ __forceinline__ void write_line(const KArgs<float> &A, const RefData<float> &ref,
+                                           const float *s_tr, float *trace_out, int el, int e, int q) {
+    using L = TraceLayout<S, float>;
     constexpr int STR = S::EPB * S::NP;
-    const int ne = A.M.ne;
     const int b0 = el * S::NP + line_node<S::D, S::P1>(J, q, 0);
     constexpr int st = J == 0 ? 1 : (J == 1 ? S::P1 : S::P1 * S::P1);
-    Real *om = trace_out + ((size_t)(2 * J) * S::NTR * ne + e) * S::NFP1 + q;
-    Real *op = trace_out + ((size_t)(2 * J + 1) * S::NTR * ne + e) * S::NFP1 + q;
-    const size_t fs = (size_t)ne * S::NFP1;
+    float *om = trace_out + L::face(e, 2 * J), *op = om + L::FACE;
+    const float2 *s2 = reinterpret_cast<const float2 *>(s_tr) + b0;
+    float2 *om2 = reinterpret_cast<float2 *>(om) + q, *op2 = reinterpret_cast<float2 *>(op) + q;
 #pragma unroll
-    for (int fld = 0; fld < S::NTR; ++fld) {
-        if (!has_trace<S>(fld, J)) continue;
-        Real v[S::P1];
-#pragma unroll
-        for (int i = 0; i < S::P1; ++i) v[i] = s_tr[fld * STR + b0 + i * st];
-        Real am = Real(0), ap = Real(0);
+    for (int p = 0; p < L::NPAIR; ++p) {
+        float2 am = make_float2(0.0f, 0.0f), ap = am;
 #pragma unroll
         for (int i = 0; i < S::P1; ++i) {
-            am = fma(ref.lm[i], v[i], am);
-            ap = fma(ref.lp[i], v[i], ap);
+            const float2 v = s2[p * STR + i * st];
+            am = __ffma2_rn(make_float2(ref.lm[i], ref.lm[i]), v, am);
+            ap = __ffma2_rn(make_float2(ref.lp[i], ref.lp[i]), v, ap);
         }
-        om[fld * fs] = am;
-        op[fld * fs] = ap;
-        if (DIFF && fld < S::NF) {
-            Real dm = Real(0), dp = Real(0);
+        om2[p * S::NFP1] = am;
+        op2[p * S::NFP1] = ap;
+    }
+#pragma unroll
+    for (int sl = 2 * L::NPAIR; sl < S::NTR; ++sl) {
+        if (!has_trace<S>(L::field(sl), J)) continue;
+        float am = 0.0f, ap = 0.0f;
+#pragma unroll
+        for (int i = 0; i < S::P1; ++i) {
+            const float v = s_tr[sl * STR + b0 + i * st];
+            am = fmaf(ref.lm[i], v, am);
+            ap = fmaf(ref.lp[i], v, ap);
+        }
+        om[sl * S::NFP1 + q] = am;
+        op[sl * S::NFP1 + q] = ap;
+    }
+    if (DIFF) {
+        const float sc = A.M.two_over_h_f[J];
+        float *dout = A.dtrace_out + ((size_t)e * S::NFACE + 2 * J) * S::NF * S::NFP1 + q;
+#pragma unroll
+        for (int fld = 0; fld < S::NF; ++fld) {
+            float dm = 0.0f, dp = 0.0f;
 #pragma unroll
             for (int i = 0; i < S::P1; ++i) {
-                dm = fma(ref.dlm[i], v[i], dm);
-                dp = fma(ref.dlp[i], v[i], dp);
+                const float v = s_tr[L::at(fld, b0 + i * st, STR)];
+                dm = fmaf(ref.dlm[i], v, dm);
+                dp = fmaf(ref.dlp[i], v, dp);
             }
-            const Real sc = mconst<Real>(A.M.two_over_h[J], A.M.two_over_h_f[J]);
-            A.dtrace_out[(((size_t)(2 * J) * S::NF + fld) * ne + e) * S::NFP1 + q] = sc * dm;
-            A.dtrace_out[(((size_t)(2 * J + 1) * S::NF + fld) * ne + e) * S::NFP1 + q] = sc * dp;
+            dout[fld * S::NFP1] = sc * dm;
+            dout[(S::NF + fld) * S::NFP1] = sc * dp;
         }
     }
 }
@@ -1101,7 +1174,7 @@ __device__ __forceinline__ void write_traces_points(const KArgs<Real> &A, const 
         for (int fld = 0; fld < S::NTR; ++fld) {
             if (!has_trace<S>(fld, j)) continue;
             const Real *v = s_tr + (size_t)fld * S::EPB * S::NP + el * S::NP;
-            trace_out[(((size_t)face * S::NTR + fld) * ne + e) * S::NFP1 + q] =
+            trace_out[TraceLayout<S, Real>::face(e, face) + fld * S::NFP1 + q] =
                 interp_face<S, Real>(v, ls, j, q);
         }
         if (DIFF) {
@@ -1110,7 +1183,7 @@ __device__ __forceinline__ void write_traces_points(const KArgs<Real> &A, const 
 #pragma unroll
             for (int fld = 0; fld < S::NF; ++fld) {
                 const Real *v = s_tr + (size_t)fld * S::EPB * S::NP + el * S::NP;
-                A.dtrace_out[(((size_t)face * S::NF + fld) * ne + e) * S::NFP1 + q] =
+                A.dtrace_out[(((size_t)e * S::NFACE + face) * S::NF + fld) * S::NFP1 + q] =
                     sc * interp_face<S, Real>(v, dls, j, q);
             }
         }
@@ -1132,10 +1205,10 @@ __device__ __forceinline__ void write_traces(const KArgs<Real> &A, const RefData
         const int e = bidx * S::EPB + el;
         if (e >= ne) continue;
         switch (j) {
-            case 0: write_line<S, Real, DIFF, 0>(A, ref, s_tr, trace_out, el, e, q); break;
-            case 1: write_line<S, Real, DIFF, 1>(A, ref, s_tr, trace_out, el, e, q); break;
+            case 0: write_line<S, DIFF, 0>(A, ref, s_tr, trace_out, el, e, q); break;
+            case 1: write_line<S, DIFF, 1>(A, ref, s_tr, trace_out, el, e, q); break;
             default:
-                write_line<S, Real, DIFF, (S::D == 3 ? 2 : 1)>(A, ref, s_tr, trace_out, el, e, q);
+                write_line<S, DIFF, (S::D == 3 ? 2 : 1)>(A, ref, s_tr, trace_out, el, e, q);
                 break;
         }
     }
@@ -1322,8 +1395,27 @@ __device__ __forceinline__ void derive_and_store(const KArgs<Real> &A, const Rea
     }
 }
 
-// The same, and the node values of the traces to s_tr.
-// STRIDE: nodes per field row of s_tr (0: the stage tile's EPB NP)
+// a node's traced values to row t of a float32 tile's s_tr (TraceLayout)
+template <class S>
+__device__ __forceinline__ void store_node(float *s_tr, int t, const float *u, float T, float rv, float pp) {
+    using L = TraceLayout<S, float>;
+    constexpr int STR = S::EPB * S::NP;
+    float v[S::NTR];
+#pragma unroll
+    for (int f = 0; f < S::NF; ++f) v[f] = u[f];
+    v[S::NF] = T;
+    v[S::NF + 1] = rv;
+    v[S::NF + 2] = pp;
+    float2 *s2 = reinterpret_cast<float2 *>(s_tr);
+#pragma unroll
+    for (int p = 0; p < L::NPAIR; ++p) s2[p * STR + t] = make_float2(v[L::field(2 * p)], v[L::field(2 * p + 1)]);
+#pragma unroll
+    for (int sl = 2 * L::NPAIR; sl < S::NTR; ++sl) s_tr[sl * STR + t] = v[L::field(sl)];
+}
+
+// Split and store, and the node values of the traces to s_tr: in the stage tile's
+// layout (TraceLayout rows of EPB NP nodes), or with STRIDE > 0 one row of
+// STRIDE nodes per field (column march).
 template <class S, typename Real, bool DIFF = false, int STRIDE = 0>
 __device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real *u, int e, int a,
                                                 int iz, Real *s_tr, int t, Real *s_red = nullptr,
@@ -1333,12 +1425,15 @@ __device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real
     if (DIFF)
         alpha_accumulate<S, Real>(A, A.ref, u, vr, a, iz * S::P1 + digit<S::D, S::P1>(a, S::VERT),
                                   s_red + 2 * (t / S::NP));
-    const int str = STRIDE > 0 ? STRIDE : S::EPB * S::NP;
+    if constexpr (STRIDE > 0) {
 #pragma unroll
-    for (int f = 0; f < S::NF; ++f) s_tr[f * str + t] = u[f];
-    s_tr[S::NF * str + t] = T;
-    s_tr[(S::NF + 1) * str + t] = rv;
-    s_tr[(S::NF + 2) * str + t] = pp;
+        for (int f = 0; f < S::NF; ++f) s_tr[f * STRIDE + t] = u[f];
+        s_tr[S::NF * STRIDE + t] = T;
+        s_tr[(S::NF + 1) * STRIDE + t] = rv;
+        s_tr[(S::NF + 2) * STRIDE + t] = pp;
+    } else {
+        store_node<S>(s_tr, t, u, T, rv, pp);
+    }
 }
 
 // Eq. (3.8) at a node at the end of a step: relax rho_m', rho_r', m, E' towards
@@ -1416,7 +1511,7 @@ __host__ __device__ constexpr size_t stage_fh_offset() {
 
 template <class S, typename Real, bool PF = false, bool DIFF = false>
 constexpr size_t stage_smem_bytes() {
-    constexpr size_t fh = (size_t)S::EPB * S::NFACE * (DIFF ? 2 * S::NF : S::NF) * S::NFP1;
+    constexpr size_t fh = (size_t)S::EPB * S::NFACE * FaceLayout<S, Real, DIFF ? 2 * S::NF : S::NF>::FACE;
     return (stage_fh_offset<S, Real, PF, DIFF>() + sizeof(Real) * fh +
             sizeof(int) * 16 * (size_t)S::EPB +  // per element: 2D neighbours, vertical index
             (DIFF ? sizeof(Real) * (size_t)S::EPB * (2 * S::NCORNER + 2) : 0) + 15) / 16 * 16;
@@ -1426,29 +1521,21 @@ constexpr size_t stage_smem_bytes() {
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // The tile's face values from the face pass's face-major buffer
-// (fbuf [faces][NFP][NFP1]; ftab [ne][2D] gives each element's faces) to
-// s_fh [EPB][2D][NFP][NFP1]: one contiguous block per face, copied
-// asynchronously in CHUNK-byte pieces by all threads; completed by
-// cp_async_wait_all.
+// (FaceLayout; ftab [ne][2D] gives each element's faces) to s_fh
+// [EPB][2D][FACE]: one contiguous block per face, copied asynchronously in
+// 16-byte pieces by all threads; completed by cp_async_wait_all.
 template <class S, typename Real, int NFP>
 __device__ __forceinline__ void cp_async_faces(const Real *fbuf, const int *ftab, Real *s_fh,
                                                int bidx, int nel) {
-    constexpr size_t FB = sizeof(Real) * (size_t)NFP * S::NFP1;   // bytes per face
-    constexpr int CHUNK = FB % 16 == 0 ? 16 : (FB % 8 == 0 ? 8 : 4);
-    constexpr int NCH = (int)(FB / CHUNK);
+    constexpr int FB = (int)sizeof(Real) * FaceLayout<S, Real, NFP>::FACE;   // bytes per face
+    constexpr int NCH = FB / 16;
     const unsigned sbase = (unsigned)__cvta_generic_to_shared(s_fh);
     const char *g = reinterpret_cast<const char *>(fbuf);
     for (int item = threadIdx.x; item < nel * S::NFACE * NCH; item += blockDim.x) {
         const int ef = item / NCH, ch = item - ef * NCH;            // (element, face), piece
-        const int fidx = __ldg(ftab + (size_t)bidx * S::EPB * S::NFACE + ef);
-        const char *src = g + (size_t)fidx * FB + (size_t)ch * CHUNK;
-        const unsigned dst = sbase + (unsigned)((size_t)ef * FB + (size_t)ch * CHUNK);
-        if (CHUNK == 16)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
-        else if (CHUNK == 8)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src));
-        else
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src));
+        const int fidx = __ldg(ftab + bidx * S::EPB * S::NFACE + ef);
+        const char *src = g + (size_t)fidx * FB + ch * 16;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sbase + 16u * item), "l"(src));
     }
     asm volatile("cp.async.commit_group;\n" ::);
 }
@@ -1556,30 +1643,24 @@ __device__ __forceinline__ void face_point(const KArgs<Real> &A, const RefData<R
                                            int e2, int nb, int iz) {
     constexpr int STR = S::EPB * S::NP;
     const MeshData &M = A.M;
-    const int ne = M.ne;
     const int s = (face & 1) ? 1 : -1;
     const Real *ls = (face & 1) ? ref.lp : ref.lm;
     Real tm[S::NTR], tp[S::NTR];
     if (sizeof(Real) == sizeof(double)) {
         // float64 form: the own trace was written with the same interpolation
         // when this state was produced; reading it back saves float64 work
-#pragma unroll
-        for (int fld = 0; fld < S::NTR; ++fld)
-            tm[fld] = has_trace<S>(fld, J)
-                          ? A.trace_in[(((size_t)face * S::NTR + fld) * ne + e2) * S::NFP1 + q]
-                          : Real(0);
+        load_traces<S, Real, J>(A.trace_in, e2, face, q, tm);
     } else {
+        using L = TraceLayout<S, Real>;
 #pragma unroll
-        for (int fld = 0; fld < S::NTR; ++fld)
-            tm[fld] = interp_face<S, Real>(s_tr + fld * STR + el2 * S::NP, ls, J, q);
+        for (int fld = 0; fld < S::NTR; ++fld) {
+            const Real *v = s_tr + L::at(fld, el2 * S::NP, STR);
+            tm[fld] = L::slot(fld) < 2 * L::NPAIR ? interp_face<S, Real, 2>(v, ls, J, q)
+                                                  : interp_face<S, Real>(v, ls, J, q);
+        }
     }
     if (nb >= 0) {
-        const int fo = 2 * J + (s > 0 ? 0 : 1);
-#pragma unroll
-        for (int fld = 0; fld < S::NTR; ++fld)
-            tp[fld] = has_trace<S>(fld, J)
-                          ? A.trace_in[(((size_t)fo * S::NTR + fld) * ne + nb) * S::NFP1 + q]
-                          : Real(0);
+        load_traces<S, Real, J>(A.trace_in, nb, 2 * J + (s > 0 ? 0 : 1), q, tp);
     } else {
 #pragma unroll
         for (int fld = 0; fld < S::NTR; ++fld) tp[fld] = tm[fld];
@@ -1602,11 +1683,12 @@ __device__ __forceinline__ void face_point(const KArgs<Real> &A, const RefData<R
         tm[fld] = lo;
     }
     lf_flux<S, Real, J>(tm, tp, brd, brm, bE, bp, M, G);
-    Real *out = s_fh + ((el2 * S::NFACE + face) * S::NF) * S::NFP1 + q;
+    using FL = FaceLayout<S, Real, S::NF>;
+    Real *out = s_fh + (el2 * S::NFACE + face) * FL::FACE;
 #pragma unroll
     for (int f = 0; f < S::NF; ++f) {
         o[f] = s > 0 ? G[f] : -G[f];
-        out[f * S::NFP1] = o[f];
+        out[FL::at(f, q)] = o[f];
     }
     if (S::RAIN && J == S::VERT && nb < 0 && A.fallout) {
         const int nh = S::D == 3 ? M.n[0] * M.n[1] : M.n[0];
@@ -1622,7 +1704,6 @@ __device__ __forceinline__ void face_point(const KArgs<Real> &A, const RefData<R
 template <class S, typename Real, int J, bool DIFF>
 __device__ __forceinline__ void face_flux(const KArgs<Real> &A, int f, int q) {
     const MeshData &M = A.M;
-    const int ne = M.ne;
     int im[3];
     {
         const int n0 = J == 0 ? M.nfn[0] : M.n[0], n1 = J == 1 ? M.nfn[1] : M.n[1];
@@ -1640,20 +1721,8 @@ __device__ __forceinline__ void face_flux(const KArgs<Real> &A, int f, int q) {
     }
     if (c < M.n[J]) e_hi = im[0] + M.n[0] * (im[1] + M.n[1] * (S::D == 3 ? im[2] : 0));
     Real tl[S::NTR], th[S::NTR];
-    if (e_lo >= 0) {
-#pragma unroll
-        for (int fld = 0; fld < S::NTR; ++fld)
-            tl[fld] = has_trace<S>(fld, J)
-                          ? A.trace_in[(((size_t)(2 * J + 1) * S::NTR + fld) * ne + e_lo) * S::NFP1 + q]
-                          : Real(0);
-    }
-    if (e_hi >= 0) {
-#pragma unroll
-        for (int fld = 0; fld < S::NTR; ++fld)
-            th[fld] = has_trace<S>(fld, J)
-                          ? A.trace_in[(((size_t)(2 * J) * S::NTR + fld) * ne + e_hi) * S::NFP1 + q]
-                          : Real(0);
-    }
+    if (e_lo >= 0) load_traces<S, Real, J>(A.trace_in, e_lo, 2 * J + 1, q, tl);
+    if (e_hi >= 0) load_traces<S, Real, J>(A.trace_in, e_hi, 2 * J, q, th);
     if (e_lo < 0) {
 #pragma unroll
         for (int fld = 0; fld < S::NTR; ++fld) tl[fld] = th[fld];
@@ -1671,11 +1740,10 @@ __device__ __forceinline__ void face_flux(const KArgs<Real> &A, int f, int q) {
         load_base<S, Real>(A.bnode, M.nzlev_node, im[S::VERT] * S::P1 + face_q_vert<S::D, S::P1>(J, q),
                            brd, brm, bE, bp);
     }
-    // face-major: [faces normal to e_0 | e_1 | e_2][NFP fields][NFP1 points],
-    // one block per face
-    constexpr int NFP = DIFF ? 2 * S::NF : S::NF;
+    // face-major: [faces normal to e_0 | e_1 | e_2], one block (FaceLayout) per face
+    using FL = FaceLayout<S, Real, DIFF ? 2 * S::NF : S::NF>;
     const size_t fg = (size_t)(J > 0 ? M.nfaces[0] : 0) + (J > 1 ? M.nfaces[1] : 0) + f;
-    Real *out = A.fbuf + fg * NFP * S::NFP1 + q;
+    Real *out = A.fbuf + fg * FL::FACE;
     Real G[S::NF];
     lf_flux<S, Real, J>(tl, th, brd, brm, bE, bp, M, G);
     if (DIFF) {
@@ -1728,20 +1796,27 @@ __device__ __forceinline__ void face_flux(const KArgs<Real> &A, int f, int q) {
             for (int fld = 0; fld < S::NF; ++fld) {
                 const Real al = (S::RAIN && fld == 2) ? ar : au;
                 const Real dl =
-                    A.dtrace_in[(((size_t)(2 * J + 1) * S::NF + fld) * ne + e_lo) * S::NFP1 + q];
-                const Real dh = A.dtrace_in[(((size_t)(2 * J) * S::NF + fld) * ne + e_hi) * S::NFP1 + q];
+                    A.dtrace_in[(((size_t)e_lo * S::NFACE + 2 * J + 1) * S::NF + fld) * S::NFP1 + q];
+                const Real dh = A.dtrace_in[(((size_t)e_hi * S::NFACE + 2 * J) * S::NF + fld) * S::NFP1 + q];
                 const Real jump = tl[fld] - th[fld];
                 G[fld] += al * (sig * jump - Real(0.5) * (dl + dh));
                 Sx[fld] = Real(0.5) * al * jump;
             }
         }
 #pragma unroll
-        for (int fld = 0; fld < S::NF; ++fld) out[(S::NF + fld) * S::NFP1] = Sx[fld];
+        for (int fld = 0; fld < S::NF; ++fld) out[FL::at(S::NF + fld, q)] = Sx[fld];
     }
     // G along +e_J: the outward flux of the element below the face; the one
     // above lifts -G (the sign sits in its lift coefficient)
+    if constexpr (FL::NPAIR > 0 && !DIFF) {
+        float2 *out2 = reinterpret_cast<float2 *>(out) + q;
 #pragma unroll
-    for (int fld = 0; fld < S::NF; ++fld) out[fld * S::NFP1] = G[fld];
+        for (int p = 0; p < FL::NPAIR; ++p) out2[p * S::NFP1] = make_float2(G[2 * p], G[2 * p + 1]);
+        if (S::NF & 1) out[FL::at(S::NF - 1, q)] = G[S::NF - 1];
+    } else {
+#pragma unroll
+        for (int fld = 0; fld < S::NF; ++fld) out[FL::at(fld, q)] = G[fld];
+    }
     if (S::RAIN && J == S::VERT && (e_lo < 0 || e_hi < 0) && A.fallout) {
         // outward normal -e_z at the bottom wall, +e_z at the top
         const int nh = S::D == 3 ? M.n[0] * M.n[1] : M.n[0];
@@ -1788,7 +1863,9 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
     constexpr int STR = S::EPB * S::NP;
     constexpr bool SHARE = tr_shares_fl<PF, DIFF>();
     constexpr int NFP = DIFF ? 2 * S::NF : S::NF;             // per face: fluxes [, symmetry terms]
-    constexpr int EB = S::NFACE * NFP * S::NFP1;              // face values of one element
+    using FL = FaceLayout<S, Real, NFP>;
+    using TL = TraceLayout<S, Real>;
+    constexpr int EB = S::NFACE * FL::FACE;                   // face values of one element
     Real *s_fl = reinterpret_cast<Real *>(smem_raw);          // nodal fluxes (fl_index)
     Real *s_tr = SHARE ? s_fl : s_fl + S::D * fl_words<S>() * STR;   // [NTR][STR]
     Real *s_fh = reinterpret_cast<Real *>(smem_raw + stage_fh_offset<S, Real, PF, DIFF>());  // [EPB][EB]
@@ -1866,16 +1943,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
         for (int f = 0; f < S::NF; ++f) R[f] = Real(0);
         // node values for the own traces (inline faces) or for the
         // derivatives of the diffusion
-        if (DIFF) {
-#pragma unroll
-            for (int f = 0; f < S::NF; ++f) s_tr[f * STR + t] = u[f];
-        } else if (!PF) {
-#pragma unroll
-            for (int f = 0; f < S::NF; ++f) s_tr[f * STR + t] = u[f];
-            s_tr[S::NF * STR + t] = T;
-            s_tr[(S::NF + 1) * STR + t] = rv;
-            s_tr[(S::NF + 2) * STR + t] = pp;
-        }
+        if (DIFF || !PF) store_node<S>(s_tr, t, u, T, rv, pp);
         // sources G (Eq. (2.11)): microphysics and gravity
         if (S::RAIN) {
             R[1] = dgm;
@@ -1904,10 +1972,10 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
                 const Real sc = mconst<Real>(M.two_over_h[j], M.two_over_h_f[j]);
 #pragma unroll
                 for (int f = 0; f < S::NF; ++f) {
-                    const Real *v = s_tr + f * STR + b0;
                     Real du = Real(0);
 #pragma unroll
-                    for (int i = 0; i < S::P1; ++i) du = fma(ref.dmat[aj][i], v[i * st], du);
+                    for (int i = 0; i < S::P1; ++i)
+                        du = fma(ref.dmat[aj][i], s_tr[TL::at(f, b0 + i * st, STR)], du);
                     const Real al = (S::RAIN && f == 2) ? ar : au;
                     s_fl[fl_index<S, STR>(j, f, t)] -= al * (sc * du);
                 }
@@ -1956,8 +2024,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
         for (int j = 0; j < S::D; ++j) {
             const int aj = digit<S::D, S::P1>(a, j);
             const int q = face_q<S::D, S::P1>(a, j);
-            const Real *fm = s_fh + ((el * S::NFACE + 2 * j) * NFP) * S::NFP1 + q;
-            const Real *fp = s_fh + ((el * S::NFACE + 2 * j + 1) * NFP) * S::NFP1 + q;
+            const Real *fm = s_fh + (el * S::NFACE + 2 * j) * FL::FACE, *fp = fm + FL::FACE;
             const Real cm = A.ref.liftm_s[j][aj], cp = A.ref.liftp_s[j][aj];
             // the low face holds the outward flux (inline) or G along +e_j,
             // which is minus this element's outward flux (face pass):
@@ -1965,17 +2032,28 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
             // alike.  Two fmas per face and field (a sum of the two products
             // first would cost a multiply and an add more).
             const Real cmo = PF ? cm : -cm;
+            if constexpr (!DIFF) {
+                // field pairs on paired fmas
+                const float2 *fm2 = reinterpret_cast<const float2 *>(fm) + q;
+                const float2 *fp2 = reinterpret_cast<const float2 *>(fp) + q;
+                const float2 c2m = make_float2(cmo, cmo), c2p = make_float2(-cp, -cp);
 #pragma unroll
-            for (int f = 0; f < S::NF; ++f)
-                R[f] = fma(cmo, fm[f * S::NFP1], fma(-cp, fp[f * S::NFP1], R[f]));
+                for (int p = 0; p < FL::NPAIR; ++p) {
+                    float2 r = make_float2(R[2 * p], R[2 * p + 1]);
+                    r = __ffma2_rn(c2m, fm2[p * S::NFP1], __ffma2_rn(c2p, fp2[p * S::NFP1], r));
+                    R[2 * p] = r.x;
+                    R[2 * p + 1] = r.y;
+                }
+            }
+#pragma unroll
+            for (int f = DIFF ? 0 : 2 * FL::NPAIR; f < S::NF; ++f)
+                R[f] = fma(cmo, fm[FL::at(f, q)], fma(-cp, fp[FL::at(f, q)], R[f]));
             if (DIFF) {
                 // symmetry term of Eq. (3.7): + (2/h_j)^2 l_a'(s)/w_a S on both faces
-                const Real *sm = fm + S::NF * S::NFP1;
-                const Real *sp = fp + S::NF * S::NFP1;
                 const Real dm = A.ref.dliftm_s[j][aj], dp = A.ref.dliftp_s[j][aj];
 #pragma unroll
                 for (int f = 0; f < S::NF; ++f)
-                    R[f] = fma(dm, sm[f * S::NFP1], fma(dp, sp[f * S::NFP1], R[f]));
+                    R[f] = fma(dm, fm[FL::at(S::NF + f, q)], fma(dp, fp[FL::at(S::NF + f, q)], R[f]));
             }
         }
         const size_t gi = (size_t)e * S::NP + a;

@@ -14,6 +14,7 @@ namespace dgm {
 template <typename Real>
 struct Launchers {
     int nf, np, nfp1, nd, ntr, epb, nt;
+    int trace_face;   // values of one face of one element in the trace buffer (TraceLayout)
     // diff: with the artificial diffusion of Eq. (3.7) (face pass only)
     cudaError_t (*prepare)(const KArgs<Real> &, bool diff, cudaStream_t);
     // pf: the stage kernel takes its face fluxes from the face pass
@@ -202,6 +203,7 @@ struct Impl {
         L.nfp1 = S::NFP1;
         L.nd = S::ND;
         L.ntr = S::NTR;
+        L.trace_face = TraceLayout<S, Real>::FACE;
         L.epb = S::EPB;
         L.nt = S::NT;
         L.prepare = &prepare;

@@ -101,7 +101,7 @@ __device__ __forceinline__ bool fx_group(const int *s_e, int *E) {
 // Shared memory of a float64 stage tile: nodal fluxes s_fl [D][NF][STR] (then
 // the node values of the traces [NTR][STR] in the same place; with diffusion
 // those have their own, as the derivatives read them first), face fluxes s_fh
-// [EPB][2D][NFP][NFP1], element indices, with diffusion the vertex
+// [EPB][2D] (FaceLayout), element indices, with diffusion the vertex
 // coefficients and alpha sums, coefficients s_cf, group exponents s_e.
 template <class S, bool DIFF>
 __host__ __device__ constexpr size_t stage64_fh_offset() {
@@ -112,7 +112,7 @@ __host__ __device__ constexpr size_t stage64_fh_offset() {
 
 template <class S, bool DIFF>
 __host__ __device__ constexpr size_t stage64_cf_offset() {
-    constexpr size_t fh = (size_t)S::EPB * S::NFACE * (DIFF ? 2 * S::NF : S::NF) * S::NFP1;
+    constexpr size_t fh = (size_t)S::EPB * S::NFACE * FaceLayout<S, double, DIFF ? 2 * S::NF : S::NF>::FACE;
     return (stage64_fh_offset<S, DIFF>() + sizeof(double) * fh + sizeof(int) * 8 * (size_t)S::EPB +
             (DIFF ? sizeof(double) * (size_t)S::EPB * (2 * S::NCORNER + 2) : 0) + 15) / 16 * 16;
 }
@@ -190,8 +190,7 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
         const int2 *x = s_x + x0;
         const double *xd = s_tr + x0;
         const int st = stride_of<S::P1>(j);
-        double *out = A.trace_out + ((size_t)(2 * j + side) * S::NTR * ne + e) * S::NFP1 + q;
-        const size_t fs = (size_t)ne * S::NFP1;
+        double *out = A.trace_out + TraceLayout<S, double>::face(e, 2 * j + side) + q;
         int2 c[S::P1];
 #pragma unroll
         for (int i = 0; i < S::P1; ++i) c[i] = s_cf[(side ? C::TP : C::TM) + i];
@@ -199,29 +198,29 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
         for (int f = 0; f < S::NTR; ++f) {
             if (!has_trace<S>(f, j)) continue;
             if (!fx_field<S>(f)) {
-                out[f * fs] = dot(s_cd + (side ? C::TP : C::TM), xd + f * STR, st);
+                out[f * S::NFP1] = dot(s_cd + (side ? C::TP : C::TM), xd + f * STR, st);
                 continue;
             }
             long long a2 = 0, a1 = 0;
 #pragma unroll
             for (int i = 0; i < S::P1; ++i) fx_mac(c[i], x[f * STR + i * st], a2, a1);
-            out[f * fs] = fx_value(a2, a1, E[f] + A.ref.q_trace);
+            out[f * S::NFP1] = fx_value(a2, a1, E[f] + A.ref.q_trace);
         }
         if constexpr (DIFF) {
-            double *dout = A.dtrace_out + ((size_t)(2 * j + side) * S::NF * ne + e) * S::NFP1 + q;
+            double *dout = A.dtrace_out + ((size_t)e * S::NFACE + 2 * j + side) * S::NF * S::NFP1 + q;
             const int qd = pick3(A.ref.q_dtrace, j);
 #pragma unroll
             for (int i = 0; i < S::P1; ++i) c[i] = s_cf[j * C::BLK + (side ? C::DTP : C::DTM) + i];
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
                 if (!fx_field<S>(f)) {
-                    dout[f * fs] = dot(s_cd + j * C::BLK + (side ? C::DTP : C::DTM), xd + f * STR, st);
+                    dout[f * S::NFP1] = dot(s_cd + j * C::BLK + (side ? C::DTP : C::DTM), xd + f * STR, st);
                     continue;
                 }
                 long long a2 = 0, a1 = 0;
 #pragma unroll
                 for (int i = 0; i < S::P1; ++i) fx_mac(c[i], x[f * STR + i * st], a2, a1);
-                dout[f * fs] = fx_value(a2, a1, E[f] + qd);
+                dout[f * S::NFP1] = fx_value(a2, a1, E[f] + qd);
             }
         }
     }
@@ -299,7 +298,8 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     using X = FxExp<S, DIFF>;
     constexpr int STR = S::EPB * S::NP;
     constexpr int NFP = DIFF ? 2 * S::NF : S::NF;             // per face: fluxes [, symmetry terms]
-    constexpr int EB = S::NFACE * NFP * S::NFP1;              // face values of one element
+    constexpr int FACE = FaceLayout<S, double, NFP>::FACE;
+    constexpr int EB = S::NFACE * FACE;                       // face values of one element
     double *s_fl = reinterpret_cast<double *>(smem_raw);
     double *s_tr = DIFF ? s_fl + S::D * S::NF * STR : s_fl;
     double *s_fh = reinterpret_cast<double *>(smem_raw + stage64_fh_offset<S, DIFF>());
@@ -464,7 +464,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
                     break;
             }
         }
-        const double *g = s_fh + ((el2 * S::NFACE + face) * NFP) * S::NFP1 + q;
+        const double *g = s_fh + (el2 * S::NFACE + face) * FACE + q;
         const int ql = pick3(A.ref.q_lift, jd);
 #pragma unroll
         for (int f = 0; f < S::NF; ++f)
@@ -501,7 +501,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
         for (int item = t; item < FACE_ITEMS; item += S::NT) {
             int jd, el2, face, q;
             if (!face_item(item, jd, el2, face, q)) continue;
-            const int k = ((el2 * S::NFACE + face) * NFP) * S::NFP1 + q;
+            const int k = (el2 * S::NFACE + face) * FACE + q;
             const int ql = pick3(A.ref.q_lift, jd), qd = DIFF ? pick3(A.ref.q_dlift, jd) : 0;
 #pragma unroll
             for (int f = 0; f < NFP; ++f) {
@@ -522,8 +522,8 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
                 const int st = stride_of<S::P1>(j);
                 const int q = face_q<S::D, S::P1>(a, j);
                 const int fl0 = j * S::NF * STR + el * S::NP + a - aj * st;
-                const int fm0 = ((el * S::NFACE + 2 * j) * NFP) * S::NFP1 + q;
-                const int2 *fl = x_fl + fl0, *fm = x_fh + fm0, *fp = fm + NFP * S::NFP1;
+                const int fm0 = (el * S::NFACE + 2 * j) * FACE + q;
+                const int2 *fl = x_fl + fl0, *fm = x_fh + fm0, *fp = fm + FACE;
                 const int2 *cf = s_cf + j * C::BLK;
                 int2 c[S::P1], cm = cf[C::LM + aj], cp = cf[C::LP + aj];
 #pragma unroll
@@ -550,7 +550,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
                 }
                 if constexpr (S::RAIN) {
                     const double *dl = s_fl + fl0 + 2 * STR, *gm = s_fh + fm0 + 2 * S::NFP1;
-                    const double *gp = gm + NFP * S::NFP1, *cd = s_cd + j * C::BLK;
+                    const double *gp = gm + FACE, *cd = s_cd + j * C::BLK;
 #pragma unroll
                     for (int i = 0; i < S::P1; ++i) rr = fma(cd[aj * S::P1 + i], dl[i * st], rr);
                     rr = fma(PF ? cd[C::LM + aj] : -cd[C::LM + aj], *gm, fma(-cd[C::LP + aj], *gp, rr));
@@ -572,8 +572,8 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
             const int st = stride_of<S::P1>(j);
             const int q = face_q<S::D, S::P1>(a, j);
             const double *fl = s_fl + j * S::NF * STR + el * S::NP + a - aj * st;
-            const double *fm = s_fh + ((el * S::NFACE + 2 * j) * NFP) * S::NFP1 + q;
-            const double *fp = fm + NFP * S::NFP1;
+            const double *fm = s_fh + (el * S::NFACE + 2 * j) * FACE + q;
+            const double *fp = fm + FACE;
             const double cm = PF ? A.ref.liftm_s[j][aj] : -A.ref.liftm_s[j][aj], cp = A.ref.liftp_s[j][aj];
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
