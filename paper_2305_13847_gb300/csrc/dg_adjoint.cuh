@@ -11,10 +11,9 @@
 //                 traces, then the split Eq. (2.8) is differentiated by the
 //                 implicit-function theorem on the active branch, giving
 //                 the adjoint of U; out = alpha out + beta w + gamma ubar.
-// The pointwise Jacobians (flux, wave-speed bound, sources, v_r) are taken
-// in forward mode with dual numbers through the same templated code the
-// forward kernels run, so the adjoint linearises exactly the computed
-// operator.  Non-smooth points take the active branch: max in Lambda, the
+// The pointwise Jacobians (flux, wave-speed bound, sources, v_r) are reverse
+// sweeps written by hand through the formulas that the forward kernels
+// evaluate, so the adjoint linearises the computed operator.  Non-smooth points take the active branch: max in Lambda, the
 // saturation min in the split, max(rho_c, 0) and max(rho_r, 0); fractional
 // powers of rain below kRainFloorLin are differentiated at the floor.
 #pragma once
@@ -22,32 +21,6 @@
 #include "dg_device.cuh"
 
 namespace dgm {
-
-// ---------------------------------------------------------------------------
-// Dual numbers (value, derivative) for forward-mode differentiation
-// ---------------------------------------------------------------------------
-struct Dual {
-    double v, d;
-    __device__ __forceinline__ Dual() : v(0.0), d(0.0) {}
-    __device__ __forceinline__ Dual(double x) : v(x), d(0.0) {}
-    __device__ __forceinline__ Dual(double x, double y) : v(x), d(y) {}
-};
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return Dual(a.v + b.v, a.d + b.d); }
-__device__ __forceinline__ Dual operator-(Dual a, Dual b) { return Dual(a.v - b.v, a.d - b.d); }
-__device__ __forceinline__ Dual operator-(Dual a) { return Dual(-a.v, -a.d); }
-__device__ __forceinline__ Dual operator*(Dual a, Dual b) { return Dual(a.v * b.v, a.d * b.v + a.v * b.d); }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-    const double q = a.v / b.v;
-    return Dual(q, (a.d - q * b.d) / b.v);
-}
-__device__ __forceinline__ Dual &operator+=(Dual &a, Dual b) { return a = a + b; }
-__device__ __forceinline__ Dual &operator-=(Dual &a, Dual b) { return a = a - b; }
-__device__ __forceinline__ bool operator>(Dual a, Dual b) { return a.v > b.v; }
-__device__ __forceinline__ bool operator<(Dual a, Dual b) { return a.v < b.v; }
-__device__ __forceinline__ bool operator!=(Dual a, Dual b) { return a.v != b.v; }
-__device__ __forceinline__ Dual fma(Dual a, Dual b, Dual c) {
-    return Dual(::fma(a.v, b.v, c.v), a.d * b.v + a.v * b.d + c.d);
-}
 
 // v_r(rho_r, rho_m) and its partial derivatives (the fractional power of
 // rho_r differentiated at max(rho_r, floor), kRainFloorLin: the powers p < 1
@@ -110,25 +83,6 @@ __device__ __forceinline__ void zero_bar(PrimBar<D> &B) {
     for (int i = 0; i < D; ++i) B.m[i] = B.u[i] = 0.0;
 }
 
-// B += W where c holds (a select per quantity, no branch)
-template <int D>
-__device__ __forceinline__ void add_bar_if(PrimBar<D> &B, const PrimBar<D> &W, bool c) {
-    B.rd += c ? W.rd : 0.0;
-    B.rm += c ? W.rm : 0.0;
-    B.rr += c ? W.rr : 0.0;
-    B.rho += c ? W.rho : 0.0;
-    B.E += c ? W.E : 0.0;
-    B.p += c ? W.p : 0.0;
-    B.T += c ? W.T : 0.0;
-    B.rv += c ? W.rv : 0.0;
-    B.vr += c ? W.vr : 0.0;
-#pragma unroll
-    for (int i = 0; i < D; ++i) {
-        B.m[i] += c ? W.m[i] : 0.0;
-        B.u[i] += c ? W.u[i] : 0.0;
-    }
-}
-
 // sign, with the derivative of |x| taken as 0 at exactly 0 (the velocity is
 // exactly 0 in a resting initial state; central differences see 0 there)
 __device__ __forceinline__ double sgn0(double x) { return x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0); }
@@ -187,10 +141,10 @@ __device__ __forceinline__ void wave_speed_vjp(const Prim<S::D, S::RAIN, double>
     const double nd = num * (cv * P.rho);
     if (!(nd > 0.0)) return;
     const double h = 0.5 * lb * num * rsqrt_nr(nd);       // c/2 times lb
-    const double a = h / (cv + R);
-    const double cvb = a - h / cv;
-    B.p += h / P.p;
-    B.rho -= h / P.rho;
+    const double a = h * recip(cv + R);
+    const double cvb = fma(-h, recip(cv), a);
+    B.p = fma(h, recip(P.p), B.p);
+    B.rho = fma(-h, P.irho, B.rho);
     B.rd += cvb * kCvd + a * kRd;
     B.rv += cvb * (kCvv - kCl) + a * kRv;
     B.rm += cvb * kCl;
@@ -242,56 +196,49 @@ __device__ __forceinline__ void flux_vjp(const double *x, double brd, double brm
 }
 
 // Sources G (Eq. (2.4), gravity) as functions of x = (U, T, rho_v, p'):
-// forward-mode Jacobian-vector products dotted with the adjoint wv.
+// xbar += wv . dG/dx.  With x_r = rho_r^(1/16), A = a - b (T - T_ref),
+// B = 1 + c x_r^3 and the deficit D = rho_vs(T) - rho_v (0 at saturation, its
+// derivatives kept),
+//   G_rm = S_ev - S_au - S_ac = A B D x_r^8 - s max(rho_c, 0) - k rho_c x_r^14,
+// G_rr = -G_rm.  About 45 float64 operations, where one dual-number pass per
+// input took about 200 (with the reciprocals below, the adjoint step of 128x64
+// order 4 went from 1.99 to 1.66 ms).
 template <class S>
-__device__ __forceinline__ void source_vjp(const double *x, double brd, double brm,
-                                           const double *wv, const MeshData &M,
-                                           const double *__restrict__ tab, double *xbar) {
+__device__ __forceinline__ void source_vjp(const double *x, double brm, const double *wv,
+                                           const MeshData &M, const double *__restrict__ tab,
+                                           double *xbar) {
     const double g = M.g;
     // gravity: G_{m_vert} = -g (rho_d' + rho_m' + rho_r'), G_E = -g m_vert
-    const double wm = wv[S::IM + S::VERT];
-    xbar[0] -= g * wm;
-    xbar[1] -= g * wm;
-    if (S::RAIN) xbar[2] -= g * wm;
+    const double gw = g * wv[S::IM + S::VERT];
+    xbar[0] -= gw;
+    xbar[1] -= gw;
+    if (S::RAIN) xbar[2] -= gw;
     xbar[S::IM + S::VERT] -= g * wv[S::IE];
     if (!S::RAIN) return;
-    // microphysics: G_rm = S_ev - S_au - S_ac, G_rr = -G_rm; inputs rho_m', rho_r', T, rho_v
     const double wg = wv[1] - wv[2];
-    const int ins[4] = {1, 2, S::NF, S::NF + 1};
-    const double rm0 = brm + x[1];
-    const bool sat = rm0 - x[S::NF + 1] > 0.0;
-    // the pieces that depend on one input only, evaluated once with their
-    // derivatives: rho_vs(T) (table) and x_r = rho_r^(1/16)
+    const double T = x[S::NF], rv = x[S::NF + 1], rc = (brm + x[1]) - rv;
     double drvs;
-    const double rvs = rho_vs_tab(x[S::NF], tab, drvs);
-    const Dual rvs1(rvs, drvs);
-    // x_r = rho_r^(1/16) = rho_r q^15, q = rho_r^(-1/16); dx_r/drho_r = x_r / (16 rho_r)
-    // at max(rho_r, floor)
-    const bool rpos = gt0(x[2]);
-    Dual xr1(0.0);
-    if (rpos) {
+    const double rvs = rho_vs_tab(T, tab, drvs);
+    const double D = rc > 0.0 ? 0.0 : rvs - rv;      // the forward value is exactly 0 at saturation
+    const double au = rc > 0.0 ? kSau : 0.0;
+    // x_r = rho_r q^15, q = rho_r^(-1/16); dx_r/drho_r = x_r / (16 rho_r) at
+    // max(rho_r, floor); all powers are 0 where there is no rain
+    double ac = 0.0;
+    if (gt0(x[2])) {
         const double q = inv_root16(x[2]);
         const double q2 = q * q, q4 = q2 * q2, q8 = q4 * q4;
         const double xr = x[2] * (q8 * q4 * q2 * q);
-        xr1 = Dual(xr, x[2] > M.rain_floor ? 0.0625 * xr * recip(x[2]) : M.rain_d16);
+        const double dx = x[2] > M.rain_floor ? 0.0625 * xr * recip(x[2]) : M.rain_d16;
+        const double x2 = xr * xr, x3 = x2 * xr, x4 = x2 * x2, x8 = x4 * x4, x13 = x8 * x4 * xr;
+        const double A = fma(-kSevB, T - kTref, kSevA), B = fma(kSevC, x3, 1.0);
+        const double Bw = wg * x8 * B;
+        xbar[S::NF] += Bw * fma(A, drvs, -kSevB * D);
+        xbar[S::NF + 1] -= Bw * A;
+        ac = kSac * xr * x13;
+        xbar[2] += wg * dx * fma(A * D * (x4 * x3), fma(3.0 * kSevC, x3, 8.0 * B), -14.0 * kSac * rc * x13);
     }
-    for (int c = 0; c < 4; ++c) {
-        const int k = ins[c];
-        const Dual rm = Dual(brm) + Dual(x[1], k == 1 ? 1.0 : 0.0);
-        const Dual T = Dual(x[S::NF], k == S::NF ? 1.0 : 0.0);
-        const Dual rv = Dual(x[S::NF + 1], k == S::NF + 1 ? 1.0 : 0.0);
-        const Dual rc = rm - rv;
-        Dual deficit = Dual(rvs1.v, k == S::NF ? rvs1.d : 0.0) - rv;
-        if (sat) deficit.v = 0.0;            // the forward value is exactly 0 at saturation
-        const Dual xr = Dual(xr1.v, k == 2 ? xr1.d : 0.0);
-        const Dual x2 = xr * xr, x3 = x2 * xr, x4 = x2 * x2, x8 = x4 * x4, x14 = x8 * x4 * x2;
-        const Dual s_ev = (Dual(kSevA) - Dual(kSevB) * (T - Dual(kTref))) *
-                          (Dual(1.0) + Dual(kSevC) * x3) * deficit * x8;
-        const Dual s_au = rc.v > 0.0 ? Dual(kSau) * rc : Dual(0.0);
-        const Dual s_ac = Dual(kSac) * rc * x14;
-        xbar[k] += wg * (s_ev - s_au - s_ac).d;
-    }
-    (void)brd;
+    xbar[1] -= wg * (au + ac);
+    xbar[S::NF + 1] += wg * (au + ac);
 }
 
 // Lax-Friedrichs face flux: adjoints of both traces at one face point.
@@ -327,7 +274,7 @@ __device__ __forceinline__ void face_vjp(const AdjArgs &A, const double *s_w, do
                              brm, bE, bp);
     }
     // adjoint of Fhat: R_a -= (2/h_J) l_a(s)/w_a Fhat(q) along the line through q
-    const double *lift = (face & 1) ? A.ref.liftp : A.ref.liftm;
+    const double *lift = (face & 1) ? A.ref.liftp_s[J] : A.ref.liftm_s[J];
     double fhb[S::NF];
 #pragma unroll
     for (int f = 0; f < S::NF; ++f) {
@@ -335,15 +282,18 @@ __device__ __forceinline__ void face_vjp(const AdjArgs &A, const double *s_w, do
 #pragma unroll
         for (int i = 0; i < S::P1; ++i)
             acc = ::fma(lift[i], s_w[f * STR + el2 * S::NP + line_node<S::D, S::P1>(J, q, i)], acc);
-        fhb[f] = -M.two_over_h[J] * acc;
+        fhb[f] = -acc;
     }
     // values: which side's wave speed is the max (forward: lam = lm > lp ? lm : lp)
     Prim<S::D, S::RAIN, double> Pm, Pp;
     make_prim<S, double>(Pm, tm, brd, brm, bE, bp, tm[S::NF], tm[S::NF + 1], tm[S::NF + 2]);
     make_prim<S, double>(Pp, tp, brd, brm, bE, bp, tp[S::NF], tp[S::NF + 1], tp[S::NF + 2]);
-    if (S::RAIN) {
-        Pm.vr = rain_velocity(Pm.rr, Pm.rm, M);
-        Pp.vr = rain_velocity(Pp.rr, Pp.rm, M);
+    RainVel rv_m = {0.0, 0.0, 0.0}, rv_p = {0.0, 0.0, 0.0};
+    if (S::RAIN && J == S::VERT) {
+        rv_m = rain_velocity_partials(Pm.rr, Pm.rm, M);
+        rv_p = rain_velocity_partials(Pp.rr, Pp.rm, M);
+        Pm.vr = rv_m.v;
+        Pp.vr = rv_p.v;
     }
     const double lmv = wave_speed<S, J, double>(Pm), lpv = wave_speed<S, J, double>(Pp);
     const bool m_active = lmv > lpv;
@@ -358,31 +308,30 @@ __device__ __forceinline__ void face_vjp(const AdjArgs &A, const double *s_w, do
         Fb[f] = hs * fhb[f];
         lb = ::fma(fhb[f], 0.5 * (tm[f] - tp[f]), lb);
     }
-    RainVel rv_m = {0.0, 0.0, 0.0}, rv_p = {0.0, 0.0, 0.0};
-    if (S::RAIN && J == S::VERT) {
-        rv_m = rain_velocity_partials(Pm.rr, Pm.rm, M);
-        rv_p = rain_velocity_partials(Pp.rr, Pp.rm, M);
-        Pm.vr = rv_m.v;
-        Pp.vr = rv_p.v;
-    }
-    PrimBar<S::D> Bm, Bp, Bw;
-    zero_bar<S::D>(Bm);
-    zero_bar<S::D>(Bp);
-    zero_bar<S::D>(Bw);
-    flux_dir_vjp<S>(Pm, J, Fb, Bm);
-    flux_dir_vjp<S>(Pp, J, Fb, Bp);
-    // the wave speed of the active side, once per lane (the side is chosen
-    // per lane by selects, so the warp runs this without divergence)
-    {
-        const Prim<S::D, S::RAIN, double> Pa = m_active ? Pm : Pp;
-        wave_speed_vjp<S, J>(Pa, lb, Bw);
-    }
-    add_bar_if<S::D>(Bm, Bw, m_active);
-    add_bar_if<S::D>(Bp, Bw, !m_active);
+    // The side whose wave speed is the max takes its derivative as well: the
+    // sides are swapped by selects into active and passive, so that the warp
+    // runs one body without divergence and the wave speed's adjoints start the
+    // active side's sums.
+    double tab[S::NTR], tpas[S::NTR];
 #pragma unroll
-    for (int k = 0; k < S::NTR; ++k) tmb[k] = tpb[k] = 0.0;
-    prim_to_inputs<S>(Pm, Bm, rv_m, tmb);
-    prim_to_inputs<S>(Pp, Bp, rv_p, tpb);
+    for (int k = 0; k < S::NTR; ++k) tab[k] = tpas[k] = 0.0;
+    {
+        const Prim<S::D, S::RAIN, double> Pa = m_active ? Pm : Pp, Pb = m_active ? Pp : Pm;
+        const RainVel ra = m_active ? rv_m : rv_p, rb = m_active ? rv_p : rv_m;
+        PrimBar<S::D> Ba, Bb;
+        zero_bar<S::D>(Ba);
+        zero_bar<S::D>(Bb);
+        wave_speed_vjp<S, J>(Pa, lb, Ba);
+        flux_dir_vjp<S>(Pa, J, Fb, Ba);
+        flux_dir_vjp<S>(Pb, J, Fb, Bb);
+        prim_to_inputs<S>(Pa, Ba, ra, tab);
+        prim_to_inputs<S>(Pb, Bb, rb, tpas);
+    }
+#pragma unroll
+    for (int k = 0; k < S::NTR; ++k) {
+        tmb[k] = m_active ? tab[k] : tpas[k];
+        tpb[k] = m_active ? tpas[k] : tab[k];
+    }
     // the jump term: d[[U]]/dU^- = 1, d[[U]]/dU^+ = -1
 #pragma unroll
     for (int f = 0; f < S::NF; ++f) {
@@ -454,15 +403,15 @@ __global__ void __launch_bounds__(S::NT) k_adj_local(AdjArgs A) {
                 double acc = 0.0;
 #pragma unroll
                 for (int i = 0; i < S::P1; ++i)
-                    acc = ::fma(A.ref.dhat[i][aj], s_w[f * STR + b0 + i * st], acc);
-                Fbar[j][f] = M.two_over_h[j] * acc;
+                    acc = ::fma(A.ref.dhat_s[j][i][aj], s_w[f * STR + b0 + i * st], acc);
+                Fbar[j][f] = acc;
             }
         }
         flux_vjp<S>(x, brd, brm, bE, bp, Fbar, M, xbar);
         double wv[S::NF];
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) wv[f] = s_w[f * STR + t];
-        source_vjp<S>(x, brd, brm, wv, M, A.rvs_tab, xbar);
+        source_vjp<S>(x, brm, wv, M, A.rvs_tab, xbar);
     }
     // face points in direction-major order (direction, element, side,
     // point), so that the lanes of a warp mostly share the face direction
