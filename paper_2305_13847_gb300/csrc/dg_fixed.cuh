@@ -57,11 +57,9 @@ __device__ __forceinline__ void fx_mac(int2 c, int2 x, long long &a2, long long 
     a1 += (long long)c.y * x.x;
 }
 
-// float64 value (rounded to nearest, ties away from zero) of an accumulator
-// pair whose terms have group exponent E (the largest exponent(x) + q over
-// the terms, with |c| < 2^q): V = a2 + a1 2^-28 counts units of 2^(E - 1080)
-__device__ __forceinline__ double fx_value(long long a2, long long a1, int E) {
-    const long long v = a2 + (a1 >> 28);
+// float64 value (rounded to nearest, ties away from zero) of a sum V that
+// counts units of 2^(E - 1080)
+__device__ __forceinline__ double fx_round(long long v, int E) {
     const long long sg = v >> 63;
     const unsigned long long m = (unsigned long long)((v ^ sg) - sg);
     const unsigned mh = (unsigned)(m >> 32), ml = (unsigned)m;
@@ -78,6 +76,17 @@ __device__ __forceinline__ double fx_value(long long a2, long long a1, int E) {
         (((unsigned long long)((h >> 11) + (ex << 20)) << 32) | __funnelshift_r(l, h, 11)) + ((l >> 10) & 1u);
     const unsigned rh = (unsigned)(r >> 32) | ((unsigned)sg & 0x80000000u);
     return h == 0u ? 0.0 : __hiloint2double((int)rh, (int)(unsigned)r);
+}
+
+// float64 value of an accumulator pair whose terms have group exponent E (the
+// largest exponent(x) + q over the terms, with |c| < 2^q)
+__device__ __forceinline__ double fx_value(long long a2, long long a1, int E) {
+    return fx_round(a2 + (a1 >> 28), E);
+}
+
+// v 2^-d towards minus infinity, d >= 0
+__device__ __forceinline__ long long fx_shift(long long v, int d) {
+    return v >> min(d, 63);
 }
 
 // s_e[k] = max(s_e[k], e[k] over the CTA) for N <= 32 groups: one warp

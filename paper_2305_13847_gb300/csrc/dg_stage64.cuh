@@ -9,11 +9,13 @@
 // and ~1000 integer operations of conversion per node, on a pipe that is
 // otherwise 4 % busy.  A group of the fixed point is one field of one tile.
 //
-// The rain density keeps float64 sums: v_r ~ rho_r^(1/8) and the adjoint's
-// rain powers see the sign and the relative size of rain many orders below
-// the tile's largest (1e-22 kg/m^3 still falls at 0.1 m/s), which a scale
-// shared by the tile does not resolve (measured: 2e-9 of the state after two
-// steps at the edge of a rain shaft, against 2e-14).
+// The rain density does not share the tile's scale: v_r ~ rho_r^(1/8) and the
+// adjoint's rain powers see the sign and the relative size of rain many orders
+// below the tile's largest (1e-22 kg/m^3 still falls at 0.1 m/s; a shared scale
+// cost 2e-9 of the state after two steps at the edge of a rain shaft, against
+// 2e-14).  Its volume and lift sums take a scale per line of each node
+// (rain_sum), which keeps 57 bits against the line's largest term as a float64
+// chain keeps 53; its short trace sums stay float64.
 #pragma once
 
 #include "dg_device.cuh"
@@ -42,14 +44,8 @@ __host__ __device__ constexpr bool fx_field(int f) {
     return !(S::RAIN && f == 2);
 }
 
-// doubles of the float64 copy of the tables (rain)
 template <class S, bool DIFF>
-__host__ __device__ constexpr int fx_doubles() {
-    return S::RAIN ? FxCoef<S, DIFF>::N : 0;
-}
-
-template <class S, bool DIFF>
-__device__ __forceinline__ void fx_coef_fill(const KArgs<double> &A, int2 *s_cf, double *s_cd) {
+__device__ __forceinline__ void fx_coef_fill(const KArgs<double> &A, int2 *s_cf) {
     using C = FxCoef<S, DIFF>;
     const RefData<double> &r = A.ref;
     for (int i = threadIdx.x; i < C::N; i += blockDim.x) {
@@ -78,7 +74,6 @@ __device__ __forceinline__ void fx_coef_fill(const KArgs<double> &A, int2 *s_cf,
             }
         }
         s_cf[i] = fx_from(v, 1022 + q);
-        if (S::RAIN) s_cd[i] = v;
     }
 }
 
@@ -125,14 +120,14 @@ struct FxExp {   // s_e: nodal fluxes, traced values, with diffusion the differe
 template <class S, bool DIFF>
 constexpr size_t stage64_smem_bytes() {
     return stage64_cf_offset<S, DIFF>() + sizeof(int2) * FxCoef<S, DIFF>::N +
-           sizeof(double) * fx_doubles<S, DIFF>() + sizeof(int) * FxExp<S, DIFF>::N;
+           sizeof(int) * FxExp<S, DIFF>::N;
 }
 
 // k_prepare: [NTR][STR] node values, alpha sums, coefficients, exponents
 template <class S, bool DIFF>
 constexpr size_t prepare64_smem_bytes() {
     return sizeof(double) * ((size_t)S::NTR * S::EPB * S::NP + 2 * S::EPB) + sizeof(int2) * FxCoef<S, DIFF>::N +
-           sizeof(double) * fx_doubles<S, DIFF>() + sizeof(int) * FxExp<S, DIFF>::N;
+           sizeof(int) * FxExp<S, DIFF>::N;
 }
 
 // Traces of the tile's node values v (U, T, rho_v, p' of this thread's node)
@@ -141,7 +136,7 @@ constexpr size_t prepare64_smem_bytes() {
 // Has barriers; the first also ends every earlier read of s_tr's memory.
 template <class S, bool DIFF>
 __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const double *v, bool valid, int bidx,
-                                               double *s_tr, const int2 *s_cf, const double *s_cd, int *s_e) {
+                                               double *s_tr, const int2 *s_cf, int *s_e) {
     using C = FxCoef<S, DIFF>;
     constexpr int STR = S::EPB * S::NP;
     const int ne = A.M.ne, t = threadIdx.x;
@@ -170,7 +165,7 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
         }
     }
     __syncthreads();
-    auto dot = [](const double *c, const double *x, int st) {   // float64 sum along a line
+    auto dot = [](const double *c, const double *x, int st) {   // float64 sum along a line (rain)
         double acc = 0.0;
 #pragma unroll
         for (int i = 0; i < S::P1; ++i) acc = fma(c[i], x[i * st], acc);
@@ -198,7 +193,7 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
         for (int f = 0; f < S::NTR; ++f) {
             if (!has_trace<S>(f, j)) continue;
             if (!fx_field<S>(f)) {
-                out[f * S::NFP1] = dot(s_cd + (side ? C::TP : C::TM), xd + f * STR, st);
+                out[f * S::NFP1] = dot(side ? A.ref.lp : A.ref.lm, xd + f * STR, st);
                 continue;
             }
             long long a2 = 0, a1 = 0;
@@ -214,7 +209,7 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
                 if (!fx_field<S>(f)) {
-                    dout[f * S::NFP1] = dot(s_cd + j * C::BLK + (side ? C::DTP : C::DTM), xd + f * STR, st);
+                    dout[f * S::NFP1] = A.M.two_over_h[j] * dot(side ? A.ref.dlp : A.ref.dlm, xd + f * STR, st);
                     continue;
                 }
                 long long a2 = 0, a1 = 0;
@@ -233,14 +228,13 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
     double *s_tr = reinterpret_cast<double *>(smem_raw);      // [NTR][STR]
     double *s_red = s_tr + S::NTR * STR;                      // [EPB][2]
     int2 *s_cf = reinterpret_cast<int2 *>(s_red + 2 * S::EPB);
-    double *s_cd = reinterpret_cast<double *>(s_cf + FxCoef<S, DIFF>::N);
-    int *s_e = reinterpret_cast<int *>(s_cd + fx_doubles<S, DIFF>());
+    int *s_e = reinterpret_cast<int *>(s_cf + FxCoef<S, DIFF>::N);
     const int t = threadIdx.x;
     const int el = t / S::NP, a = t - el * S::NP;
     const int e = bidx * S::EPB + el;
     const bool valid = t < STR && e < A.M.ne;
     double v[S::NTR];
-    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
+    fx_coef_fill<S, DIFF>(A, s_cf);
     if (t < FxExp<S, DIFF>::N) s_e[t] = 0;
     if (DIFF && t < 2 * S::EPB) s_red[t] = 0.0;
     dependents_wait();
@@ -257,7 +251,7 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
                                         vert_index<S::D>(A.M, e) * S::P1 + digit<S::D, S::P1>(a, S::VERT),
                                         s_red + 2 * el);
     }
-    write_traces64<S, DIFF>(A, v, valid, bidx, s_tr, s_cf, s_cd, s_e);
+    write_traces64<S, DIFF>(A, v, valid, bidx, s_tr, s_cf, s_e);
     if (DIFF) alpha_store<S, double>(A, s_red, bidx);
 }
 
@@ -288,6 +282,84 @@ __device__ __forceinline__ void flux_all(const Prim<S::D, S::RAIN, double> &P, d
     }
 }
 
+// Volume and lift terms of field f at a node as float64 sums
+template <class S, bool PF, bool DIFF, int FACE>
+__device__ __noinline__ double line_sums(const KArgs<double> &A, const double *s_fl, const double *s_fh,
+                                         int el, int a, int f) {
+    constexpr int STR = S::EPB * S::NP;
+    double r = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < S::D; ++j) {
+        const int aj = digit<S::D, S::P1>(a, j), st = stride_of<S::P1>(j);
+        const double *fl = s_fl + (j * S::NF + f) * STR + el * S::NP + a - aj * st;
+        const double *fm = s_fh + (el * S::NFACE + 2 * j) * FACE + f * S::NFP1 + face_q<S::D, S::P1>(a, j);
+        const double *fp = fm + FACE;
+        const double cm = PF ? A.ref.liftm_s[j][aj] : -A.ref.liftm_s[j][aj], cp = A.ref.liftp_s[j][aj];
+        for (int i = 0; i < S::P1; ++i) r = fma(A.ref.dhat_s[j][aj][i], fl[i * st], r);
+        r = fma(cm, *fm, fma(-cp, *fp, r));
+        if (DIFF)
+            r = fma(A.ref.dliftm_s[j][aj], fm[S::NF * S::NFP1],
+                    fma(A.ref.dliftp_s[j][aj], fp[S::NF * S::NFP1], r));
+    }
+    return r;
+}
+
+// Volume and lift terms of the rain density at a node: per direction the P1
+// flux values (fl0, stride st) and the two face values (fm0, face block FACE)
+// as fixed point with the line's own exponent, the three sums aligned to the
+// largest.  About 500 integer operations for 21 float64 fmas: at the 32 : 1
+// rate of the pipes half the time, on the one that has room.  ok is cleared
+// where a value leaves the fixed-point range.
+template <class S, bool PF, bool DIFF, int FACE>
+__device__ __forceinline__ double rain_sum(const KArgs<double> &A, const double *s_fl, const double *s_fh,
+                                           const int2 *s_cf, int el, int a, bool &ok) {
+    using C = FxCoef<S, DIFF>;
+    constexpr int STR = S::EPB * S::NP;
+    constexpr int NL = S::P1 + (DIFF ? 4 : 2);
+    long long v = 0;
+    int E = kFxMinE;
+#pragma unroll 1
+    for (int j = 0; j < S::D; ++j) {
+        const int aj = digit<S::D, S::P1>(a, j), st = stride_of<S::P1>(j);
+        const double *fl = s_fl + (j * S::NF + 2) * STR + el * S::NP + a - aj * st;
+        const double *gm = s_fh + (el * S::NFACE + 2 * j) * FACE + 2 * S::NFP1 + face_q<S::D, S::P1>(a, j);
+        const double *gp = gm + FACE;
+        const int2 *cf = s_cf + j * C::BLK;
+        const int qv = A.ref.q_vol[j], ql = A.ref.q_lift[j], qd = DIFF ? A.ref.q_dlift[j] : 0;
+        double x[NL];
+        int Ej = kFxMinE;
+#pragma unroll
+        for (int i = 0; i < S::P1; ++i) {
+            x[i] = fl[i * st];
+            Ej = max(Ej, fx_expo(x[i]) + qv);
+        }
+        x[S::P1] = *gp;
+        x[S::P1 + 1] = *gm;
+        Ej = max(Ej, max(fx_expo(*gp), fx_expo(*gm)) + ql);
+        if constexpr (DIFF) {
+            x[S::P1 + 2] = gp[S::NF * S::NFP1];
+            x[S::P1 + 3] = gm[S::NF * S::NFP1];
+            Ej = max(Ej, max(fx_expo(x[S::P1 + 2]), fx_expo(x[S::P1 + 3])) + qd);
+        }
+        ok = ok && Ej <= kFxMaxE;
+        long long a2 = 0, a1 = 0;
+#pragma unroll
+        for (int i = 0; i < S::P1; ++i) fx_mac(cf[aj * S::P1 + i], fx_from(x[i], Ej - qv), a2, a1);
+        // -(high face), +(low face along +e_j) or -(outward flux)
+        const int2 cp = cf[C::LP + aj], cm = cf[C::LM + aj];
+        fx_mac(make_int2(-cp.x, -cp.y), fx_from(x[S::P1], Ej - ql), a2, a1);
+        fx_mac(PF ? cm : make_int2(-cm.x, -cm.y), fx_from(x[S::P1 + 1], Ej - ql), a2, a1);
+        if constexpr (DIFF) {
+            fx_mac(cf[C::DLP + aj], fx_from(x[S::P1 + 2], Ej - qd), a2, a1);
+            fx_mac(cf[C::DLM + aj], fx_from(x[S::P1 + 3], Ej - qd), a2, a1);
+        }
+        const int En = max(E, Ej);
+        v = fx_shift(v, En - E) + fx_shift(a2 + (a1 >> 28), En - Ej);
+        E = En;
+    }
+    return fx_round(v, E);
+}
+
 // One tile of EPB consecutive elements (tile index bidx) of the stage kernel:
 // stage_block's phases (dg_device.cuh) with fixed-point contractions.  Every
 // thread of the CTA takes part.
@@ -307,8 +379,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     double *s_al = reinterpret_cast<double *>(s_info + 8 * S::EPB);        // DIFF: [EPB][2][NCORNER]
     double *s_red = s_al + S::EPB * 2 * S::NCORNER;                        // DIFF: [EPB][2]
     int2 *s_cf = reinterpret_cast<int2 *>(smem_raw + stage64_cf_offset<S, DIFF>());
-    double *s_cd = reinterpret_cast<double *>(s_cf + C::N);
-    int *s_e = reinterpret_cast<int *>(s_cd + fx_doubles<S, DIFF>());
+    int *s_e = reinterpret_cast<int *>(s_cf + C::N);
     int2 *x_fl = reinterpret_cast<int2 *>(s_fl), *x_fh = reinterpret_cast<int2 *>(s_fh);
     int2 *x_tr = reinterpret_cast<int2 *>(s_tr);
     const MeshData &M = A.M;
@@ -320,7 +391,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     const bool valid = (t < STR) && (e < ne);
     const size_t gi = (size_t)e * S::NP + a;
 
-    fx_coef_fill<S, DIFF>(A, s_cf, s_cd);
+    fx_coef_fill<S, DIFF>(A, s_cf);
     if (t < X::N) s_e[t] = 0;
     dependents_wait();
     // the node's state and derived fields: loads issued first, so that their
@@ -513,7 +584,6 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
         __syncthreads();
         if (valid) {
             long long a2[S::NF], a1[S::NF];
-            double rr = 0.0;      // rain density
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) a2[f] = a1[f] = 0;
 #pragma unroll 1
@@ -548,43 +618,19 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
                         fx_mac(dm, fm[(S::NF + f) * S::NFP1], a2[f], a1[f]);
                     }
                 }
-                if constexpr (S::RAIN) {
-                    const double *dl = s_fl + fl0 + 2 * STR, *gm = s_fh + fm0 + 2 * S::NFP1;
-                    const double *gp = gm + FACE, *cd = s_cd + j * C::BLK;
-#pragma unroll
-                    for (int i = 0; i < S::P1; ++i) rr = fma(cd[aj * S::P1 + i], dl[i * st], rr);
-                    rr = fma(PF ? cd[C::LM + aj] : -cd[C::LM + aj], *gm, fma(-cd[C::LP + aj], *gp, rr));
-                    if constexpr (DIFF)
-                        rr = fma(cd[C::DLM + aj], gm[S::NF * S::NFP1],
-                                 fma(cd[C::DLP + aj], gp[S::NF * S::NFP1], rr));
-                }
             }
 #pragma unroll
-            for (int f = 0; f < S::NF; ++f) R[f] = fx_field<S>(f) ? fx_value(a2[f], a1[f], ex[f]) : rr;
+            for (int f = 0; f < S::NF; ++f) R[f] = fx_field<S>(f) ? fx_value(a2[f], a1[f], ex[f]) : 0.0;
+            if constexpr (S::RAIN) {
+                bool ok = true;
+                R[2] = rain_sum<S, PF, DIFF, FACE>(A, s_fl, s_fh, s_cf, el, a, ok);
+                if (!ok) R[2] = line_sums<S, PF, DIFF, FACE>(A, s_fl, s_fh, el, a, 2);
+            }
         }
     } else if (valid) {
         // values outside the fixed-point range (infinities, NaN): float64 sums
 #pragma unroll
-        for (int f = 0; f < S::NF; ++f) R[f] = 0.0;
-#pragma unroll 1
-        for (int j = 0; j < S::D; ++j) {
-            const int aj = digit<S::D, S::P1>(a, j);
-            const int st = stride_of<S::P1>(j);
-            const int q = face_q<S::D, S::P1>(a, j);
-            const double *fl = s_fl + j * S::NF * STR + el * S::NP + a - aj * st;
-            const double *fm = s_fh + (el * S::NFACE + 2 * j) * FACE + q;
-            const double *fp = fm + FACE;
-            const double cm = PF ? A.ref.liftm_s[j][aj] : -A.ref.liftm_s[j][aj], cp = A.ref.liftp_s[j][aj];
-#pragma unroll
-            for (int f = 0; f < S::NF; ++f) {
-#pragma unroll
-                for (int i = 0; i < S::P1; ++i) R[f] = fma(A.ref.dhat_s[j][aj][i], fl[f * STR + i * st], R[f]);
-                R[f] = fma(cm, fm[f * S::NFP1], fma(-cp, fp[f * S::NFP1], R[f]));
-                if (DIFF)
-                    R[f] = fma(A.ref.dliftm_s[j][aj], fm[(S::NF + f) * S::NFP1],
-                               fma(A.ref.dliftp_s[j][aj], fp[(S::NF + f) * S::NFP1], R[f]));
-            }
-        }
+        for (int f = 0; f < S::NF; ++f) R[f] = line_sums<S, PF, DIFF, FACE>(A, s_fl, s_fh, el, a, f);
     }
 
     // ---- phase 4: sources G (Eq. (2.11): microphysics and gravity), then
@@ -618,7 +664,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
         }
     }
     if (MODE == MODE_STAGE) {
-        write_traces64<S, DIFF>(A, v, valid, bidx, s_tr, s_cf, s_cd, s_e);
+        write_traces64<S, DIFF>(A, v, valid, bidx, s_tr, s_cf, s_e);
         if (DIFF) alpha_store<S, double>(A, s_red, bidx);
     }
 }
