@@ -54,7 +54,8 @@ struct AdjArgs {
     MeshData M;
     RefData<double> ref;
     const double *U;        // state (ABI layout)
-    const double *derived;  // T, rho_v, p' (, G, v_r) of U
+    const double *derived;  // T, 1/rho, p' (, G, v_r) of U
+    const double *rv;       // rho_v of U
     const double *trace;    // traces of U (TraceLayout)
     const double *bnode, *bface;  // base tables
     const double *rvs_tab;  // rho_vs Taylor table (dg_math.cuh)
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(S::NT) k_adj_local(AdjArgs A) {
             s_w[f * STR + t] = A.w[f * nodes + gi];
         }
         x[S::NF] = A.derived[gi];
-        x[S::NF + 1] = A.derived[nodes + gi];
+        x[S::NF + 1] = A.rv[gi];
         x[S::NF + 2] = A.derived[2 * nodes + gi];
         const int lev = vert_index<S::D>(M, e) * S::P1 + digit<S::D, S::P1>(a, S::VERT);
         load_base<S, double>(A.bnode, M.nzlev_node, lev, brd, brm, bE, bp);
@@ -540,7 +541,7 @@ __global__ void k_adj_gather(AdjArgs A) {
         const int lev = vert_index<S::D>(M, e) * S::P1 + digit<S::D, S::P1>(a, S::VERT);
         double brd, brm, bE, bp;
         load_base<S, double>(A.bnode, M.nzlev_node, lev, brd, brm, bE, bp);
-        split_vjp<S>(u, brd, brm, bE, A.derived[gi], A.derived[nodes + gi], xb[S::NF], xb[S::NF + 1],
+        split_vjp<S>(u, brd, brm, bE, A.derived[gi], A.rv[gi], xb[S::NF], xb[S::NF + 1],
                      xb[S::NF + 2], A.rvs_tab, xb);
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) {
@@ -576,7 +577,7 @@ __global__ void __launch_bounds__(kRedThreads) k_cloud(AdjArgs A, double *partia
         const int lev = vert_index<S::D>(M, e) * S::P1 + digit<S::D, S::P1>(a, S::VERT);
         double brd, brm, bE, bp;
         load_base<S, double>(A.bnode, M.nzlev_node, lev, brd, brm, bE, bp);
-        const double T = A.derived[gi], rv = A.derived[nodes + gi];
+        const double T = A.derived[gi], rv = A.rv[gi];
         acc += W * (brm + u[1] - rv);
         ub[1] += W;                                       // d rho_c / d rho_m'
         split_vjp<S>(u, brd, brm, bE, T, rv, 0.0, -W, 0.0, A.rvs_tab, ub);

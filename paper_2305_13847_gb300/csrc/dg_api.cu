@@ -302,23 +302,21 @@ int copy_chunk(dg_ctx *c, int k, void *dst, const void *src, cudaMemcpyKind kind
 
 // split and traces of state U into trace buffer tb; ntiles > 0: only the
 // element tiles [tile0, tile0 + ntiles)
-// keep_rv: the derived fields hold rho_v for the adjoint kernels
 template <typename Real>
 int do_prepare(dg_ctx *c, const Launchers<Real> *L, const RefData<Real> &ref, const void *U, int tb,
-               int tile0, int ntiles, bool keep_rv) {
+               int tile0, int ntiles) {
     KArgs<Real> A = base_args<Real>(c, ref);
     A.Uin = (const Real *)U;
     A.trace_out = (Real *)c->trace[tb];
     A.dtrace_out = (Real *)c->dtrace[tb];
     A.tile0 = tile0;
     A.ntiles = ntiles;
-    A.keep_rv = keep_rv;
     return cuda_status(L->prepare(A, c->diff, c->stream));
 }
 
-int prepare(dg_ctx *c, const void *U, int tb, int tile0 = 0, int ntiles = 0, bool keep_rv = false) {
-    return c->fp32 ? do_prepare<float>(c, c->L32, c->ref32, U, tb, tile0, ntiles, keep_rv)
-                   : do_prepare<double>(c, c->L64, c->ref64, U, tb, tile0, ntiles, keep_rv);
+int prepare(dg_ctx *c, const void *U, int tb, int tile0 = 0, int ntiles = 0) {
+    return c->fp32 ? do_prepare<float>(c, c->L32, c->ref32, U, tb, tile0, ntiles)
+                   : do_prepare<double>(c, c->L64, c->ref64, U, tb, tile0, ntiles);
 }
 
 // Upload of a host state in kChunks chunks of whole element tiles: the
@@ -434,7 +432,8 @@ void release(dg_ctx *c) {
     void *ptrs[] = {c->U[0], c->U[1], c->derived, c->trace[0], c->trace[1], c->bnode_d,
                     c->bface_d, c->bnode_r, c->bface_r, c->flags, c->partials, c->rvs_tab,
                     c->adjX[0], c->adjX[1], c->adjX[2], c->adjL[0], c->adjL[1], c->adjL[2],
-                    c->ubar_part, c->tadj, c->bsplit, c->fbuf, c->ftab, c->alphaK, c->alphaV,
+                    c->ubar_part, c->tadj, c->adjRv[0], c->adjD[1], c->adjD[2], c->adjD[3],
+                    c->adjT[1], c->adjT[2], c->adjT[3], c->adjRv[1], c->adjRv[2], c->adjRv[3], c->bsplit, c->fbuf, c->ftab, c->alphaK, c->alphaV,
                     c->dtrace[0], c->dtrace[1], c->sponge, c->fallout};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -542,27 +541,89 @@ int upload_base(dg_ctx *c, const double *node_tab, const double *face_tab) {
     return DG_OK;
 }
 
+// Scratch of the adjoint entry points, on first use.  Set 0 (derived fields,
+// rho_v and traces of one state) uses the context's own buffers.  A reversed
+// step keeps the sets of all four stage states, so that none is split twice
+// (four of five k_prepare launches less; the adjoint step of 128x64 order 4:
+// 1.65 -> 1.51 ms); where the device has no room for the other three it does
+// with set 0 and splits each state again.
 int ensure_adjoint(dg_ctx *c) {
     if (c->ubar_part) return DG_OK;
     const size_t state = (size_t)c->nodes * c->nf * sizeof(double);
     const size_t trace = (size_t)2 * c->cfg.dim * c->ne * c->trace_face * sizeof(double);
+    const size_t derived = (size_t)c->nodes * c->nd * sizeof(double), rv = (size_t)c->nodes * sizeof(double);
     int st = DG_OK;
-    for (int i = 0; i < 3 && st == DG_OK; ++i) st = alloc(c, &c->adjX[i], state);
-    for (int i = 0; i < 3 && st == DG_OK; ++i) st = alloc(c, (void **)&c->adjL[i], state);
-    if (st == DG_OK) st = alloc(c, (void **)&c->tadj, trace);
+    c->adjD[0] = (double *)c->derived;
+    c->adjT[0] = (double *)c->trace[0];
+    if (!c->adjRv[0]) st = alloc(c, (void **)&c->adjRv[0], rv);
+    for (int i = 0; i < 3 && st == DG_OK; ++i)
+        if (!c->adjX[i]) st = alloc(c, &c->adjX[i], state);
+    for (int i = 0; i < 3 && st == DG_OK; ++i)
+        if (!c->adjL[i]) st = alloc(c, (void **)&c->adjL[i], state);
+    if (st == DG_OK && !c->tadj) st = alloc(c, (void **)&c->tadj, trace);
     if (st == DG_OK) st = alloc(c, (void **)&c->ubar_part, (size_t)c->nodes * c->ntr * sizeof(double));
+    if (st != DG_OK) return st;
+    for (int k = 1; k < 4 && st == DG_OK; ++k) {
+        st = alloc(c, (void **)&c->adjD[k], derived);
+        if (st == DG_OK) st = alloc(c, (void **)&c->adjT[k], trace);
+        if (st == DG_OK) st = alloc(c, (void **)&c->adjRv[k], rv);
+    }
+    if (st != DG_OK) {
+        for (int k = 1; k < 4; ++k) {
+            c->device_bytes -= (c->adjD[k] ? derived : 0) + (c->adjT[k] ? trace : 0) + (c->adjRv[k] ? rv : 0);
+            for (double **p : {&c->adjD[k], &c->adjT[k], &c->adjRv[k]}) {
+                if (*p) cudaFree(*p);
+                *p = nullptr;
+            }
+        }
+    }
+    return DG_OK;
+}
+
+// split and traces of U with rho_v, for the adjoint kernels, into set k
+int prepare_adjoint(dg_ctx *c, const void *U, int k) {
+    c->derived_valid = false;
+    KArgs<double> A = base_args<double>(c, c->ref64);
+    A.Uin = (const double *)U;
+    A.derived_out = c->adjD[k];
+    A.rv_out = c->adjRv[k];
+    A.trace_out = c->adjT[k];
+    return cuda_status(c->L64->prepare(A, false, c->stream));
+}
+
+// one stage of the step being reversed: from the state of set k to that of
+// set k + 1, whose derived fields, rho_v and traces it leaves there
+int stage_adjoint(dg_ctx *c, const void *Uin, const void *Un, void *Uout, int k, double alpha, double beta,
+                  double gdt) {
+    KArgs<double> A = base_args<double>(c, c->ref64);
+    A.fallout = nullptr;
+    A.Uin = (const double *)Uin;
+    A.Un = (const double *)Un;
+    A.Uout = (double *)Uout;
+    A.derived = c->adjD[k];
+    A.derived_out = c->adjD[k + 1];
+    A.rv_out = c->adjRv[k + 1];
+    A.trace_in = c->adjT[k];
+    A.trace_out = c->adjT[k + 1];
+    A.alpha = alpha;
+    A.beta = beta;
+    A.gdt = gdt;
+    const bool pf = use_face_pass(c);
+    int st = pf ? cuda_status(c->L64->face(A, false, c->stream)) : DG_OK;
+    if (st == DG_OK) st = cuda_status(c->L64->stage(A, MODE_STAGE, pf, false, c->stream));
     return st;
 }
 
-AdjArgs adj_args(const dg_ctx *c, const void *U, const double *w, double *out, double alpha,
+AdjArgs adj_args(const dg_ctx *c, const void *U, int k, const double *w, double *out, double alpha,
                  double beta, double gamma) {
     AdjArgs A;
     std::memset(&A, 0, sizeof(A));
     A.M = c->M;
     A.ref = c->ref64;
     A.U = (const double *)U;
-    A.derived = (const double *)c->derived;
-    A.trace = (const double *)c->trace[0];
+    A.derived = c->adjD[k];
+    A.rv = c->adjRv[k];
+    A.trace = c->adjT[k];
     A.bnode = c->bnode_d;
     A.bface = c->bface_d;
     A.rvs_tab = c->rvs_tab;
@@ -576,13 +637,11 @@ AdjArgs adj_args(const dg_ctx *c, const void *U, const double *w, double *out, d
     return A;
 }
 
-// out = alpha out + beta w + gamma (dR/dU (U))^T w
-int rhs_adjoint_into(dg_ctx *c, const void *U, const double *w, double *out, double alpha,
+// out = alpha out + beta w + gamma (dR/dU (U))^T w, the split and traces of U
+// in set k
+int rhs_adjoint_into(dg_ctx *c, const void *U, int k, const double *w, double *out, double alpha,
                      double beta, double gamma) {
-    c->derived_valid = false;
-    int st = prepare(c, U, 0, 0, 0, true);
-    if (st != DG_OK) return st;
-    AdjArgs A = adj_args(c, U, w, out, alpha, beta, gamma);
+    AdjArgs A = adj_args(c, U, k, w, out, alpha, beta, gamma);
     if (c->LA->local(A, c->stream) != cudaSuccess) return DG_ECUDA;
     if (c->LA->gather(A, c->stream) != cudaSuccess) return DG_ECUDA;
     return DG_OK;
@@ -1120,7 +1179,9 @@ int dg_rhs_adjoint(dg_ctx *c, const void *U, const double *w, double *ubar) {
     DeviceGuard dg(c->device);
     int st = ensure_adjoint(c);
     if (st != DG_OK) return st;
-    return rhs_adjoint_into(c, U, w, ubar, 0.0, 0.0, 1.0);
+    st = prepare_adjoint(c, U, 0);
+    if (st != DG_OK) return st;
+    return rhs_adjoint_into(c, U, 0, w, ubar, 0.0, 0.0, 1.0);
 }
 
 int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1, double *lam_n) {
@@ -1135,22 +1196,36 @@ int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1
     // forward stages of SSPRK(4,3) from U^n (Shu-Osher form):
     //   U1 = U^n + dt/2 R(U^n); U2 = U1 + dt/2 R(U1); U3 = 2/3 U^n + 1/3 U2 + dt/6 R(U2)
     void *X1 = c->adjX[0], *X2 = c->adjX[1], *X3 = c->adjX[2];
-    st = prepare(c, U_n, 0);
-    if (st == DG_OK) st = stage(c, MODE_STAGE, U_n, U_n, X1, 0, 0.0, 1.0, 0.5 * dt);
-    if (st == DG_OK) st = stage(c, MODE_STAGE, X1, X1, X2, 1, 0.0, 1.0, 0.5 * dt);
-    if (st == DG_OK) st = stage(c, MODE_STAGE, X2, U_n, X3, 0, 2.0 / 3.0, 1.0 / 3.0, dt / 6.0);
+    const void *X[4] = {U_n, X1, X2, X3};
+    const bool sets = c->adjRv[3] != nullptr;    // every stage state's split and traces kept
+    if (sets) {
+        st = prepare_adjoint(c, U_n, 0);
+        if (st == DG_OK) st = stage_adjoint(c, U_n, U_n, X1, 0, 0.0, 1.0, 0.5 * dt);
+        if (st == DG_OK) st = stage_adjoint(c, X1, X1, X2, 1, 0.0, 1.0, 0.5 * dt);
+        if (st == DG_OK) st = stage_adjoint(c, X2, U_n, X3, 2, 2.0 / 3.0, 1.0 / 3.0, dt / 6.0);
+    } else {
+        st = prepare(c, U_n, 0);
+        if (st == DG_OK) st = stage(c, MODE_STAGE, U_n, U_n, X1, 0, 0.0, 1.0, 0.5 * dt);
+        if (st == DG_OK) st = stage(c, MODE_STAGE, X1, X1, X2, 1, 0.0, 1.0, 0.5 * dt);
+        if (st == DG_OK) st = stage(c, MODE_STAGE, X2, U_n, X3, 0, 2.0 / 3.0, 1.0 / 3.0, dt / 6.0);
+    }
     if (st != DG_OK) return st;
+    // out = alpha out + beta w + gamma (dR/dU (X_k))^T w
+    auto reverse = [&](int k, const double *w, double *out, double alpha, double beta, double gamma) {
+        const int p = sets ? DG_OK : prepare_adjoint(c, X[k], 0);
+        return p != DG_OK ? p : rhs_adjoint_into(c, X[k], sets ? k : 0, w, out, alpha, beta, gamma);
+    };
     // reverse: U^{n+1} = U3 + dt/2 R(U3)
     double *l3 = c->adjL[0], *l2 = c->adjL[1], *l1 = c->adjL[2];
-    st = rhs_adjoint_into(c, X3, lam_np1, l3, 0.0, 1.0, 0.5 * dt);            // l3 = l + dt/2 J3^T l
-    if (st == DG_OK) st = rhs_adjoint_into(c, X2, l3, l2, 0.0, 1.0 / 3.0, dt / 6.0);  // l2
-    if (st == DG_OK) st = rhs_adjoint_into(c, X1, l2, l1, 0.0, 1.0, 0.5 * dt);        // l1
+    st = reverse(3, lam_np1, l3, 0.0, 1.0, 0.5 * dt);                       // l3 = l + dt/2 J3^T l
+    if (st == DG_OK) st = reverse(2, l3, l2, 0.0, 1.0 / 3.0, dt / 6.0);     // l2
+    if (st == DG_OK) st = reverse(1, l2, l1, 0.0, 1.0, 0.5 * dt);           // l1
     if (st != DG_OK) return st;
     // lam_n = 2/3 l3 + l1 + dt/2 J(U^n)^T l1
     const size_t bytes = (size_t)c->nodes * c->nf * sizeof(double);
     if (cudaMemcpyAsync(lam_n, l3, bytes, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
         return DG_ECUDA;
-    return rhs_adjoint_into(c, U_n, l1, lam_n, 2.0 / 3.0, 1.0, 0.5 * dt);
+    return reverse(0, l1, lam_n, 2.0 / 3.0, 1.0, 0.5 * dt);
 }
 
 int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
@@ -1158,10 +1233,13 @@ int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     if (c->fp32 || !c->LA) return DG_ENOTIMPL;
     if (!c->base_set) return DG_ESTATE;
     DeviceGuard dg(c->device);
-    c->derived_valid = false;
-    int st = prepare(c, U, 0, 0, 0, true);
+    c->adjD[0] = (double *)c->derived;
+    c->adjT[0] = (double *)c->trace[0];
+    int st = DG_OK;
+    if (!c->adjRv[0]) st = alloc(c, (void **)&c->adjRv[0], (size_t)c->nodes * sizeof(double));
+    if (st == DG_OK) st = prepare_adjoint(c, U, 0);
     if (st != DG_OK) return st;
-    AdjArgs A = adj_args(c, U, nullptr, dJdU, 0.0, 0.0, 1.0);
+    AdjArgs A = adj_args(c, U, 0, nullptr, dJdU, 0.0, 0.0, 1.0);
     if (c->LA->cloud(A, c->partials, c->nred, c->stream) != cudaSuccess) return DG_ECUDA;
     std::vector<double> h(c->nred);
     if (cudaMemcpyAsync(h.data(), c->partials, sizeof(double) * c->nred, cudaMemcpyDeviceToHost,

@@ -52,6 +52,9 @@ struct dg_ctx {
     void *adjX[3] = {nullptr, nullptr, nullptr};
     double *adjL[3] = {nullptr, nullptr, nullptr};
     double *ubar_part = nullptr, *tadj = nullptr;
+    // derived fields, rho_v and traces of the stage states of a reversed step
+    // (0: of U^n; all or none of 1 .. 3: see ensure_adjoint)
+    double *adjD[4] = {}, *adjT[4] = {}, *adjRv[4] = {};
     int nred = 0;
     std::vector<double> z_node, z_face;
     // host uploads (dg_set_state): the copies of one chunk go to up_stream

@@ -140,7 +140,7 @@ struct KArgs {
     const Real *Uin;       // state the operator is evaluated on (ABI layout)
     const Real *Un;        // U^n for the stage combination (may equal Uin)
     Real *Uout;            // MODE_RHS: dU/dt; MODE_STAGE: new stage state
-    Real *derived;         // [ND][nodes]: T, rho_v (float64: 1/rho, see keep_rv), p' [, G_rm, v_r]
+    Real *derived;         // [ND][nodes]: T, rho_v (float64: 1/rho), p' [, G_rm, v_r]
     const Real *trace_in;  // traces of Uin (TraceLayout)
     Real *trace_out;       // traces of Uout (MODE_STAGE)
     const Real *bnode;     // base at node levels [4][nzlev_node]: rho_d, rho_m, E, p
@@ -169,7 +169,9 @@ struct KArgs {
     // (ntiles 0: all), so that an upload is split while its chunks arrive
     // and a download starts while the last stage still runs
     int tile0, ntiles;
-    int keep_rv;           // float64 k_prepare: derived field 1 is rho_v (adjoint), else 1/rho
+    // float64: the derived fields of the state produced (null: `derived`, in
+    // place) and its rho_v (null: not stored; the adjoint kernels read it)
+    Real *derived_out, *rv_out;
 };
 
 // float64 value of a storage-type value (widen: integer pipe)
@@ -1381,17 +1383,21 @@ __device__ __forceinline__ void derive_and_store(const KArgs<Real> &A, const Rea
         gm = (Real)nd.gm;
         vr = (Real)nd.vr;
     }
-    A.derived[gi] = T;
-    // the float64 stage kernel's nodal flux takes 1/rho, which the split has
-    // formed, and not rho_v (its traces carry that); the adjoint takes rho_v
-    if (sizeof(Real) == sizeof(double))
-        A.derived[nodes + gi] = A.keep_rv ? rv : (Real)nd.irho;
-    else
-        A.derived[nodes + gi] = rv;
-    A.derived[2 * nodes + gi] = pp;
+    Real *out = A.derived;
+    if (sizeof(Real) == sizeof(double)) {
+        // the float64 stage kernel's nodal flux takes 1/rho, which the split
+        // has formed, and not rho_v (its traces carry that)
+        if (A.derived_out) out = A.derived_out;
+        out[nodes + gi] = (Real)nd.irho;
+        if (A.rv_out) A.rv_out[gi] = rv;
+    } else {
+        out[nodes + gi] = rv;
+    }
+    out[gi] = T;
+    out[2 * nodes + gi] = pp;
     if (S::RAIN) {
-        A.derived[3 * nodes + gi] = gm;
-        A.derived[4 * nodes + gi] = vr;
+        out[3 * nodes + gi] = gm;
+        out[4 * nodes + gi] = vr;
     }
 }
 
