@@ -1219,12 +1219,12 @@ __device__ __forceinline__ void write_traces(const KArgs<Real> &A, const RefData
 // ---------------------------------------------------------------------------
 // Artificial diffusion helpers (Section 3.5)
 // ---------------------------------------------------------------------------
-// weight W_a |K|/2^d of node a times |u|^2 and |u - v_r e_z|^2, added to the
-// element's sums s_red[0..1] (shared memory)
+// weight W_a |K|/2^d of node a times |u|^2 and |u - v_r e_z|^2, to the node's
+// place t in s_red [2][EPB NP] (shared memory; alpha_store adds them up)
 template <class S, typename Real>
 __device__ __forceinline__ void alpha_accumulate(const KArgs<Real> &A, const RefData<Real> &ref,
                                                  const Real *u, Real vr, int a, int lev,
-                                                 Real *s_red) {
+                                                 Real *s_red, int t) {
     const int nl = A.M.nzlev_node;
     const Real rho = (A.bnode[lev] + u[0]) + (A.bnode[nl + lev] + u[1]) + (S::RAIN ? u[2] : Real(0));
     const Real inv = recip(rho);
@@ -1239,20 +1239,38 @@ __device__ __forceinline__ void alpha_accumulate(const KArgs<Real> &A, const Ref
         const Real ur = (j == S::VERT) ? uj - vr : uj;
         w2r = fma(ur, ur, w2r);
     }
-    atomicAdd(&s_red[0], wq * w2u);
-    if (S::RAIN) atomicAdd(&s_red[1], wq * w2r);
+    s_red[t] = wq * w2u;
+    if (S::RAIN) s_red[S::EPB * S::NP + t] = wq * w2r;
 }
 
-// alpha_K = alpha_pre ||w||_{0,K} from the element sums (threads t < EPB)
+// alpha_K = alpha_pre ||w||_{0,K}: the sums over each element's nodes by groups
+// of G lanes, in a fixed order.  (A float64 atomicAdd on shared memory is a
+// compare-and-swap loop, one retry per contending thread: 128 float64
+// operations per node of the 415 of the order 4 stage kernel with diffusion.)
+// Called by whole CTAs after a barrier behind alpha_accumulate.
 template <class S, typename Real>
 __device__ __forceinline__ void alpha_store(const KArgs<Real> &A, const Real *s_red, int bidx) {
-    const int t = threadIdx.x;
-    if (t < S::EPB) {
-        const int e = bidx * S::EPB + t;
-        if (e < A.M.ne) {
+    constexpr int G = S::NP <= 4 ? 4 : (S::NP <= 8 ? 8 : (S::NP <= 16 ? 16 : 32));
+    constexpr int PASS = S::NT / G;                    // elements per pass
+    const int lane = threadIdx.x % G;
+    for (int e0 = 0; e0 < S::EPB; e0 += PASS) {
+        const int el = e0 + threadIdx.x / G, e = bidx * S::EPB + el;
+        const bool ok = el < S::EPB && e < A.M.ne;
+        Real su = Real(0), sr = Real(0);
+        if (ok)
+            for (int a = lane; a < S::NP; a += G) {
+                su += s_red[el * S::NP + a];
+                if (S::RAIN) sr += s_red[(S::EPB + el) * S::NP + a];
+            }
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) {
+            su += __shfl_xor_sync(0xffffffffu, su, off);
+            if (S::RAIN) sr += __shfl_xor_sync(0xffffffffu, sr, off);
+        }
+        if (ok && lane == 0) {
             const Real pre = mconst<Real>(A.M.alpha_pre, A.M.alpha_pre_f);
-            A.alphaK[e] = pre * sqrt(s_red[2 * t]);
-            A.alphaK[A.M.ne + e] = S::RAIN ? pre * sqrt(s_red[2 * t + 1]) : Real(0);
+            A.alphaK[e] = pre * sqrt(su);
+            A.alphaK[A.M.ne + e] = S::RAIN ? pre * sqrt(sr) : Real(0);
         }
     }
 }
@@ -1429,8 +1447,7 @@ __device__ __forceinline__ void split_and_store(const KArgs<Real> &A, const Real
     Real T, rv, pp, vr;
     derive_and_store<S, Real>(A, u, e, a, iz, Tprev, T, rv, pp, vr);
     if (DIFF)
-        alpha_accumulate<S, Real>(A, A.ref, u, vr, a, iz * S::P1 + digit<S::D, S::P1>(a, S::VERT),
-                                  s_red + 2 * (t / S::NP));
+        alpha_accumulate<S, Real>(A, A.ref, u, vr, a, iz * S::P1 + digit<S::D, S::P1>(a, S::VERT), s_red, t);
     if constexpr (STRIDE > 0) {
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) s_tr[f * STRIDE + t] = u[f];
@@ -1463,16 +1480,12 @@ __global__ void __launch_bounds__(S::NT) k_prepare(KArgs<Real> A) {
     dependents_go();
     dependents_wait();
     Real *s_tr = reinterpret_cast<Real *>(smem_raw);  // [NTR][EPB*NP]
-    Real *s_red = s_tr + S::NTR * S::EPB * S::NP;    // [EPB][2]
+    Real *s_red = s_tr + S::NTR * S::EPB * S::NP;    // DIFF: [2][EPB NP]
     const int t = threadIdx.x;
     const int el = t / S::NP, a = t - el * S::NP;
     const int bidx = blockIdx.x + A.tile0;
     const int e = bidx * S::EPB + el;
     const bool valid = (t < S::EPB * S::NP) && (e < A.M.ne);
-    if (DIFF) {
-        if (t < 2 * S::EPB) s_red[t] = Real(0);
-        __syncthreads();
-    }
     if (valid) {
         const size_t nodes = (size_t)A.M.ne * S::NP;
         const size_t gi = (size_t)e * S::NP + a;
@@ -1496,7 +1509,7 @@ constexpr int MODE_STAGE = 1;
 // values for the traces s_tr [NTR][EPB NP], outward face fluxes s_fh
 // [EPB][2D][NFP][NFP1] (with diffusion NFP = 2 NF: the fluxes, then the
 // symmetry terms), per-element indices, with diffusion the element's vertex
-// coefficients [EPB][2][2^D] and its alpha sums [EPB][2].  s_tr is needed
+// coefficients [EPB][2][2^D] and its nodes' alpha terms [2][EPB NP].  s_tr is needed
 // before the volume phase only when the inline form interpolates its own
 // traces in the face phase, or with diffusion (the derivatives of the node
 // values); otherwise it is filled after the volume phase and shares s_fl.
@@ -1520,7 +1533,7 @@ constexpr size_t stage_smem_bytes() {
     constexpr size_t fh = (size_t)S::EPB * S::NFACE * FaceLayout<S, Real, DIFF ? 2 * S::NF : S::NF>::FACE;
     return (stage_fh_offset<S, Real, PF, DIFF>() + sizeof(Real) * fh +
             sizeof(int) * 16 * (size_t)S::EPB +  // per element: 2D neighbours, vertical index
-            (DIFF ? sizeof(Real) * (size_t)S::EPB * (2 * S::NCORNER + 2) : 0) + 15) / 16 * 16;
+            (DIFF ? sizeof(Real) * (size_t)S::EPB * (2 * S::NCORNER + 2 * S::NP) : 0) + 15) / 16 * 16;
 }
 
 // completes the asynchronous copies issued by this thread
@@ -1877,7 +1890,7 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
     Real *s_fh = reinterpret_cast<Real *>(smem_raw + stage_fh_offset<S, Real, PF, DIFF>());  // [EPB][EB]
     int *s_info = reinterpret_cast<int *>(s_fh + S::EPB * EB);                            // [EPB][16]
     Real *s_al = reinterpret_cast<Real *>(s_info + 16 * S::EPB);        // DIFF: [EPB][2][NCORNER]
-    Real *s_red = s_al + S::EPB * 2 * S::NCORNER;                       // DIFF: [EPB][2]
+    Real *s_red = s_al + S::EPB * 2 * S::NCORNER;                       // DIFF: [2][EPB NP]
     const MeshData &M = A.M;
     const int ne = M.ne;
     const size_t nodes = (size_t)ne * S::NP;
@@ -1922,10 +1935,6 @@ __device__ __forceinline__ void stage_block(const KArgs<Real> &A, const RefData<
             }
             s_info[t * 16 + 6] = im[S::VERT];
             if (DIFF) alpha_corners<S, Real>(A, im, s_al + t * 2 * S::NCORNER);
-        }
-        if (DIFF) {
-            s_red[2 * t] = Real(0);
-            s_red[2 * t + 1] = Real(0);
         }
     }
     __syncthreads();

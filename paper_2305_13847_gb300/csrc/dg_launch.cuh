@@ -72,7 +72,7 @@ struct Impl {
     template <bool DIFF>
     static constexpr size_t prep_smem() {
         if constexpr (F64) return prepare64_smem_bytes<S, DIFF>();
-        else return sizeof(Real) * ((size_t)S::NTR * S::EPB * S::NP + 2 * S::EPB);
+        else return sizeof(Real) * (size_t)(S::NTR + (DIFF ? 2 : 0)) * S::EPB * S::NP;
     }
     template <bool PF, bool DIFF>
     static constexpr size_t stage_smem() {

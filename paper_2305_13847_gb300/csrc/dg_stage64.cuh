@@ -97,7 +97,7 @@ __device__ __forceinline__ bool fx_group(const int *s_e, int *E) {
 // the node values of the traces [NTR][STR] in the same place; with diffusion
 // those have their own, as the derivatives read them first), face fluxes s_fh
 // [EPB][2D] (FaceLayout), element indices, with diffusion the vertex
-// coefficients and alpha sums, coefficients s_cf, group exponents s_e.
+// coefficients and alpha terms, coefficients s_cf, group exponents s_e.
 template <class S, bool DIFF>
 __host__ __device__ constexpr size_t stage64_fh_offset() {
     constexpr size_t FL = (size_t)S::D * S::NF;
@@ -109,7 +109,7 @@ template <class S, bool DIFF>
 __host__ __device__ constexpr size_t stage64_cf_offset() {
     constexpr size_t fh = (size_t)S::EPB * S::NFACE * FaceLayout<S, double, DIFF ? 2 * S::NF : S::NF>::FACE;
     return (stage64_fh_offset<S, DIFF>() + sizeof(double) * fh + sizeof(int) * 8 * (size_t)S::EPB +
-            (DIFF ? sizeof(double) * (size_t)S::EPB * (2 * S::NCORNER + 2) : 0) + 15) / 16 * 16;
+            (DIFF ? sizeof(double) * (size_t)S::EPB * (2 * S::NCORNER + 2 * S::NP) : 0) + 15) / 16 * 16;
 }
 
 template <class S, bool DIFF>
@@ -123,10 +123,10 @@ constexpr size_t stage64_smem_bytes() {
            sizeof(int) * FxExp<S, DIFF>::N;
 }
 
-// k_prepare: [NTR][STR] node values, alpha sums, coefficients, exponents
+// k_prepare: [NTR][STR] node values, alpha terms, coefficients, exponents
 template <class S, bool DIFF>
 constexpr size_t prepare64_smem_bytes() {
-    return sizeof(double) * ((size_t)S::NTR * S::EPB * S::NP + 2 * S::EPB) + sizeof(int2) * FxCoef<S, DIFF>::N +
+    return sizeof(double) * (size_t)(S::NTR + (DIFF ? 2 : 0)) * S::EPB * S::NP + sizeof(int2) * FxCoef<S, DIFF>::N +
            sizeof(int) * FxExp<S, DIFF>::N;
 }
 
@@ -226,8 +226,8 @@ template <class S, bool DIFF>
 __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx, unsigned char *smem_raw) {
     constexpr int STR = S::EPB * S::NP;
     double *s_tr = reinterpret_cast<double *>(smem_raw);      // [NTR][STR]
-    double *s_red = s_tr + S::NTR * STR;                      // [EPB][2]
-    int2 *s_cf = reinterpret_cast<int2 *>(s_red + 2 * S::EPB);
+    double *s_red = s_tr + S::NTR * STR;                      // DIFF: [2][STR]
+    int2 *s_cf = reinterpret_cast<int2 *>(s_red + (DIFF ? 2 * STR : 0));
     int *s_e = reinterpret_cast<int *>(s_cf + FxCoef<S, DIFF>::N);
     const int t = threadIdx.x;
     const int el = t / S::NP, a = t - el * S::NP;
@@ -236,7 +236,6 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
     double v[S::NTR];
     fx_coef_fill<S, DIFF>(A, s_cf);
     if (t < FxExp<S, DIFF>::N) s_e[t] = 0;
-    if (DIFF && t < 2 * S::EPB) s_red[t] = 0.0;
     dependents_wait();
     __syncthreads();
     if (valid) {
@@ -249,7 +248,7 @@ __device__ __forceinline__ void prepare_block64(const KArgs<double> &A, int bidx
         if (DIFF)
             alpha_accumulate<S, double>(A, A.ref, v, vr, a,
                                         vert_index<S::D>(A.M, e) * S::P1 + digit<S::D, S::P1>(a, S::VERT),
-                                        s_red + 2 * el);
+                                        s_red, t);
     }
     write_traces64<S, DIFF>(A, v, valid, bidx, s_tr, s_cf, s_e);
     if (DIFF) alpha_store<S, double>(A, s_red, bidx);
@@ -377,7 +376,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     double *s_fh = reinterpret_cast<double *>(smem_raw + stage64_fh_offset<S, DIFF>());
     int *s_info = reinterpret_cast<int *>(s_fh + S::EPB * EB);             // inline: [EPB][8] neighbours
     double *s_al = reinterpret_cast<double *>(s_info + 8 * S::EPB);        // DIFF: [EPB][2][NCORNER]
-    double *s_red = s_al + S::EPB * 2 * S::NCORNER;                        // DIFF: [EPB][2]
+    double *s_red = s_al + S::EPB * 2 * S::NCORNER;                        // DIFF: [2][STR]
     int2 *s_cf = reinterpret_cast<int2 *>(smem_raw + stage64_cf_offset<S, DIFF>());
     int *s_e = reinterpret_cast<int *>(s_cf + C::N);
     int2 *x_fl = reinterpret_cast<int2 *>(s_fl), *x_fh = reinterpret_cast<int2 *>(s_fh);
@@ -422,7 +421,6 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
             }
             if (DIFF) alpha_corners<S, double>(A, im, s_al + t * 2 * S::NCORNER);
         }
-        if (DIFF && t < 2 * S::EPB) s_red[t] = 0.0;
     }
     const int iz = e / (S::D == 3 ? M.n[0] * M.n[1] : M.n[0]);
 
@@ -660,7 +658,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
             derive_and_store<S, double>(A, v, e, a, iz, dT, v[S::NF], v[S::NF + 1], v[S::NF + 2], vr);
             if (DIFF)
                 alpha_accumulate<S, double>(A, A.ref, v, vr, a, iz * S::P1 + digit<S::D, S::P1>(a, S::VERT),
-                                            s_red + 2 * el);
+                                            s_red, t);
         }
     }
     if (MODE == MODE_STAGE) {
