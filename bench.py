@@ -494,6 +494,10 @@ def _roofline(info, word, t_total, steps, peak, peak_kind, traffic=(None, None))
 FP64_FMA_PER_SM_CLK = 2
 
 
+# items of fp64_flops_per_node that the kernels sum on the integer pipe
+INTEGER_PIPE_ITEMS = ("volume", "lift", "traces")
+
+
 def fp64_flops_per_node(dim, order, nf, rain):
     """Algorithmic float64 operations per node and SSPRK stage of the
     sum-factorised DG stage (fma = 2, any other operation 1, a transcendental
@@ -536,6 +540,11 @@ def fp64_alu_roofline(info, w, t_total, steps, sm_count, sm_mhz, probe_tflops, h
            "traffic": hbm["traffic"], "traffic_source": hbm["traffic_source"],
            "algorithmic_flops_per_node": fpn,
            "flops_per_node_items": items, "avg_launch_ms": 1000.0 * launch_s,
+           # the linear contractions run as fixed point on the integer pipe, beside
+           # the FP64 pipe, so frac may pass 1; this is the fraction of the rest
+           "integer_pipe_items": list(INTEGER_PIPE_ITEMS),
+           "frac_without_integer_items":
+               achieved / peak * (1.0 - sum(items[k] for k in INTEGER_PIPE_ITEMS) / fpn),
            "hbm": {k: hbm[k] for k in ("achieved", "peak", "peak_kind", "unit", "frac",
                                        "algorithmic_bytes_per_launch")}}
     if probe_tflops:

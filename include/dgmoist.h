@@ -91,20 +91,19 @@ typedef struct dg_config {
                            the perturbation variables T - T_bar, rho_v - rho_v_bar
                            against a float64 split of the base state (no
                            cancellation, so float32 suffices there);
-                           DG_FP64_FFC: float64 state and arithmetic as
-                           DG_FP64, except that the stage kernel's volume
-                           term and lift (the sum-factorised contractions of
-                           Eq. (3.2) and the facet term of Eq. (3.3)) are
-                           compensated float32-pair sums (error-free
-                           transformations, ~2^-48 relative to the sum of the
-                           terms' magnitudes) on the float32 pipe, which runs
-                           64x the float64 rate on GB300; not in the paper */
+                           DG_FP64_FFC: the same as DG_FP64.  (It asked for
+                           the linear contractions as float32-pair sums, when
+                           DG_FP64 took them on the float64 pipe; both now
+                           sum them in 57-bit fixed point on the integer
+                           pipe, faster and closer than the pairs.) */
     double g;           /* gravity in m/s^2 (the paper does not print it; 9.81 usual) */
     double rho_w;       /* water density in the rain speed: <= 0 takes the paper's
                            rho_w = rho_v + rho_c + rho_r; > 0 a constant (kg/m^3) */
     int faces;          /* where the Lax-Friedrichs face fluxes of a stage are
                            evaluated: DG_FACES_AUTO (0) the library's choice (the
-                           face pass); DG_FACES_INLINE in the stage kernel, by both
+                           face pass; inline for meshes of about a wave of
+                           element tiles, where a second launch costs more
+                           than the doubled face work); DG_FACES_INLINE in the stage kernel, by both
                            elements of a face; DG_FACES_PASS once per face point in a
                            separate face kernel (an extra flux buffer of
                            n_f (k+1)^(d-1) values per face); DG_FACES_COLUMN (float32
@@ -329,8 +328,7 @@ int dg_rhs_noalloc_status(long long counts[2], void *cuda_stream);
  * bounded and leaves it exact wherever rho_r >= 1e-12.  Uses the context's
  * derived-field and trace buffers (the next dg_step re-derives them).
  * DG_ENOTIMPL for float32 contexts (DG_FP32_BULK, DG_FP32_PERT);
- * asynchronous.  In a DG_FP64_FFC context the adjoint kernels are the
- * float64 ones. */
+ * asynchronous. */
 int dg_rhs_adjoint(dg_ctx *ctx, const void *U, const double *w, double *ubar);
 
 /* Adjoint of one SSPRK(4,3) step of size dt from the state U_n (device,
@@ -339,9 +337,10 @@ int dg_rhs_adjoint(dg_ctx *ctx, const void *U, const double *w, double *ubar);
  * stages are then reversed (Remark 3.1, Shu-Osher form) with dg_rhs_adjoint.
  * lam_np1, lam_n: device float64, ABI layout, distinct.  Allocates six
  * state-sized and one trace-sized scratch buffers in the context on first
- * use.  DG_ENOTIMPL for float32 contexts (DG_FP32_BULK, DG_FP32_PERT);
- * asynchronous.  A DG_FP64_FFC context recomputes the stage states with its
- * own stage kernel (float-float contractions). */
+ * use, and for the three intermediate states a set of traces, derived fields
+ * and rho_v each where the device has the memory (without them each state is
+ * split a second time).  DG_ENOTIMPL for float32 contexts (DG_FP32_BULK,
+ * DG_FP32_PERT); asynchronous. */
 int dg_adjoint_step(dg_ctx *ctx, double dt, const void *U_n, const double *lam_np1,
                     double *lam_n);
 
@@ -473,8 +472,8 @@ void dg_ensemble_free(dg_ensemble *ens);
  *                  float64 compares x > 0, x > 1.5, x < 1.5, |x| <= 1.5,
  *                  isfinite(x), max(|x|, 1.5) against those of the library's
  *                  bit-pattern compares;
- *                  FF_SPLIT writes hi + lo of the float32 pair of
- *                  DG_FP64_FFC (in float64) and, beside it, x itself;
+ *                  FF_SPLIT writes hi + lo of the float32 pair of x (in
+ *                  float64) and, beside it, x itself;
  *   out[2n .. 4n)  for FF_SPLIT the pair's hi and CUDA's float32 rounding
  *                  of x; for RHO_VS / RHO_VS_F32 / RHO_VS_BULK the derivative
  *                  d rho_vs / dT, the library's (RHO_VS_BULK: the float32

@@ -207,30 +207,16 @@ __device__ __forceinline__ double inv_root8(double r) {
     return k == 0 ? v : v * pow2(16 * k);
 }
 
-// ---------------------------------------------------------------------------
-// Compensated float32-pair ("double-float") sums for the float64 form with
-// float-float contractions (DG_FP64_FFC).  GB300 issues float64 at 1/64 of
-// the float32 rate, so a linear contraction sum_i c_i x_i of float64 values
-// costs less as error-free float32 transformations (Dekker's product by fma,
-// Knuth's TwoSum) than as float64 fmas.
-//
-// ff_split(x) = (hi, lo): hi = x rounded to float32 (as narrow), lo = x - hi
-// to 24 bits.  For x in the float32 normal range, x - hi is the float64
-// mantissa's dropped 29 bits (less 2^29 when hi rounded up) times
-// 2^(e - 1075), so lo is built from them by integer operations (leading bit,
-// shift, exponent; truncated) with no float64 subtraction.  Then
-// |x - hi - lo| <= 2^-47 |x| + 2^-126 (lo is flushed to zero below the
-// float32 normal range, which happens only for |x| below ~1e-28); other x
-// (zero, tiny, huge, not finite) take narrow(x - widen(hi)).
-// ff_madd(c, x, s, e): s + e += c x for pairs c, x.  The product c.hi x.hi is
-// split exactly by one fma, the cross terms c.hi x.lo + c.lo x.hi are added
-// to that error, c.lo x.lo (< 2^-48 |c x|) is dropped, and s + p is a TwoSum
-// whose rounding error goes to e.  The sum of n terms is then within about
-// n 2^-47 of sum |c_i x_i| (Ogita, Rump and Oishi, "Accurate sum and dot
-// product", SIAM J. Sci. Comput. 26 (2005), Dot2), against n 2^-53 in
-// float64.  The _rn intrinsics keep the compiler from fusing the
-// transformation's multiplies and adds into fmas, which would break it.
-// ---------------------------------------------------------------------------
+// A float64 as a pair of float32: ff_split(x) = (hi, lo), hi = x rounded to
+// float32 (as narrow), lo = x - hi to 24 bits.  For x in the float32 normal
+// range, x - hi is the float64 mantissa's dropped 29 bits (less 2^29 when hi
+// rounded up) times 2^(e - 1075), so lo is built from them by integer
+// operations (leading bit, shift, exponent; truncated) with no float64
+// subtraction.  Then |x - hi - lo| <= 2^-47 |x| + 2^-126 (lo is flushed to zero
+// below the float32 normal range, which happens only for |x| below ~1e-28);
+// other x (zero, tiny, huge, not finite) take narrow(x - widen(hi)).  Offered
+// by dg_selftest_math; the kernels' own contractions are fixed point
+// (dg_fixed.cuh), which is both faster and 10 bits closer.
 __device__ __forceinline__ float2 ff_split(double x) {
     const unsigned hx = (unsigned)__double2hiint(x), lx = (unsigned)__double2loint(x);
     const unsigned mag = hx & 0x7fffffffu, e = mag >> 20;
@@ -251,50 +237,6 @@ __device__ __forceinline__ float2 ff_split(double x) {
     return make_float2(h, __uint_as_float((up ? sx ^ 0x80000000u : sx) | ((unsigned)ef << 23) |
                                           (m & 0x7fffffu)));
 }
-
-__device__ __forceinline__ void ff_madd(float2 c, float2 x, float &s, float &e) {
-    const float p = __fmul_rn(c.x, x.x);
-    float q = __fmaf_rn(c.x, x.x, -p);          // c.hi x.hi - p, exact
-    q = __fmaf_rn(c.x, x.y, q);
-    q = __fmaf_rn(c.y, x.x, q);
-    const float t = __fadd_rn(s, p);
-    const float bp = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-    s = t;
-    e = __fadd_rn(e, __fadd_rn(err, q));
-}
-
-// Two lanes at once on the paired float32 instructions (fma.rn.f32x2 and
-// friends): lane by lane the same operations as ff_madd, so the same
-// results.  The coefficient c = (c.hi, c.lo) is the same in both lanes; the
-// error terms are accumulated negated (r = p - c.hi x.hi - cross terms) so
-// that every fma takes the coefficient's negation instead of a negated sum.
-__device__ __forceinline__ float2 ff_sub2(float2 a, float2 b) {
-    unsigned long long ra, rb, rd;
-    ra = ((unsigned long long)__float_as_uint(a.y) << 32) | __float_as_uint(a.x);
-    rb = ((unsigned long long)__float_as_uint(b.y) << 32) | __float_as_uint(b.x);
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
-    return make_float2(__uint_as_float((unsigned)rd), __uint_as_float((unsigned)(rd >> 32)));
-}
-
-__device__ __forceinline__ void ff_madd2(float2 c, float2 xh, float2 xl, float2 &s, float2 &e) {
-    const float2 ch = make_float2(c.x, c.x), nh = make_float2(-c.x, -c.x),
-                 nl = make_float2(-c.y, -c.y);
-    const float2 p = __fmul2_rn(ch, xh);
-    float2 r = __ffma2_rn(nh, xh, p);           // p - c.hi x.hi, exact
-    r = __ffma2_rn(nh, xl, r);
-    r = __ffma2_rn(nl, xh, r);
-    const float2 t = __fadd2_rn(s, p);
-    const float2 bp = ff_sub2(t, s);
-    const float2 err = __fadd2_rn(ff_sub2(s, ff_sub2(t, bp)), ff_sub2(p, bp));
-    s = t;
-    e = __fadd2_rn(e, ff_sub2(err, r));
-}
-
-// the float64 value of s + e (both exact in float64; one rounding)
-__device__ __forceinline__ double ff_value(float s, float e) { return widen(s) + widen(e); }
-
-__device__ __forceinline__ float2 ff_neg(float2 c) { return make_float2(-c.x, -c.y); }
 
 // x != 0 (either sign of zero is zero), for kernel parameters
 __device__ __forceinline__ bool nonzero(double x) {

@@ -85,7 +85,7 @@ __global__ void k_selftest_math(int fn, const double *__restrict__ x, double *__
                 break;
             }
             case DG_MATH_FF_SPLIT: {
-                // the float32 pair of DG_FP64_FFC: hi + lo next to x, and hi
+                // the float32 pair of ff_split: hi + lo next to x, and hi
                 // next to the hardware conversion
                 const float2 p = ff_split(v);
                 ours = (double)p.x + (double)p.y;
