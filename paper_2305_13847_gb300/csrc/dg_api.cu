@@ -580,13 +580,14 @@ int ensure_adjoint(dg_ctx *c) {
     return DG_OK;
 }
 
-// split and traces of U with rho_v, for the adjoint kernels, into set k
-int prepare_adjoint(dg_ctx *c, const void *U, int k) {
+// split and traces of U with rho_v, for the adjoint kernels, into set k (rho_v
+// into `rv` if given)
+int prepare_adjoint(dg_ctx *c, const void *U, int k, double *rv = nullptr) {
     c->derived_valid = false;
     KArgs<double> A = base_args<double>(c, c->ref64);
     A.Uin = (const double *)U;
     A.derived_out = c->adjD[k];
-    A.rv_out = c->adjRv[k];
+    A.rv_out = rv ? rv : c->adjRv[k];
     A.trace_out = c->adjT[k];
     return cuda_status(c->L64->prepare(A, false, c->stream));
 }
@@ -1235,11 +1236,12 @@ int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     DeviceGuard dg(c->device);
     c->adjD[0] = (double *)c->derived;
     c->adjT[0] = (double *)c->trace[0];
-    int st = DG_OK;
-    if (!c->adjRv[0]) st = alloc(c, (void **)&c->adjRv[0], (size_t)c->nodes * sizeof(double));
-    if (st == DG_OK) st = prepare_adjoint(c, U, 0);
+    // rho_v passes through the first field of dJdU: k_cloud reads a node's
+    // before it writes that node's gradient
+    const int st = prepare_adjoint(c, U, 0, dJdU);
     if (st != DG_OK) return st;
     AdjArgs A = adj_args(c, U, 0, nullptr, dJdU, 0.0, 0.0, 1.0);
+    A.rv = dJdU;
     if (c->LA->cloud(A, c->partials, c->nred, c->stream) != cudaSuccess) return DG_ECUDA;
     std::vector<double> h(c->nred);
     if (cudaMemcpyAsync(h.data(), c->partials, sizeof(double) * c->nred, cudaMemcpyDeviceToHost,
