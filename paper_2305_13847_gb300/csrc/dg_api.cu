@@ -581,7 +581,8 @@ int ensure_adjoint(dg_ctx *c) {
 }
 
 // split and traces of U with rho_v, for the adjoint kernels, into set k (rho_v
-// into `rv` if given)
+// into `rv` if given: derive_and_store writes it after 1/rho, so it may take
+// the place of 1/rho, which the adjoint kernels do not read)
 int prepare_adjoint(dg_ctx *c, const void *U, int k, double *rv = nullptr) {
     c->derived_valid = false;
     KArgs<double> A = base_args<double>(c, c->ref64);
@@ -1236,12 +1237,13 @@ int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     DeviceGuard dg(c->device);
     c->adjD[0] = (double *)c->derived;
     c->adjT[0] = (double *)c->trace[0];
-    // rho_v passes through the first field of dJdU: k_cloud reads a node's
-    // before it writes that node's gradient
-    const int st = prepare_adjoint(c, U, 0, dJdU);
+    // rho_v in the place of 1/rho: dJdU may be U itself (k_cloud reads a node's
+    // state before it writes that node's gradient), so nothing passes through it
+    double *rv = c->adjD[0] + c->nodes;
+    const int st = prepare_adjoint(c, U, 0, rv);
     if (st != DG_OK) return st;
     AdjArgs A = adj_args(c, U, 0, nullptr, dJdU, 0.0, 0.0, 1.0);
-    A.rv = dJdU;
+    A.rv = rv;
     if (c->LA->cloud(A, c->partials, c->nred, c->stream) != cudaSuccess) return DG_ECUDA;
     std::vector<double> h(c->nred);
     if (cudaMemcpyAsync(h.data(), c->partials, sizeof(double) * c->nred, cudaMemcpyDeviceToHost,
