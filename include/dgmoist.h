@@ -335,14 +335,22 @@ int dg_rhs_adjoint(dg_ctx *ctx, const void *U, const double *w, double *ubar);
  * ABI layout, float64): lam_n = (dU^{n+1}/dU^n)^T lam_np1.  The three
  * intermediate stage states are recomputed from U_n inside the call; the
  * stages are then reversed (Remark 3.1, Shu-Osher form) with dg_rhs_adjoint.
- * lam_np1, lam_n: device float64, ABI layout, distinct.  Allocates six
- * state-sized and one trace-sized scratch buffers in the context on first
- * use, and for the three intermediate states a set of traces, derived fields
- * and rho_v each where the device has the memory (without them each state is
- * split a second time).  DG_ENOTIMPL for float32 contexts (DG_FP32_BULK,
- * DG_FP32_PERT); asynchronous. */
+ * lam_np1, lam_n: device float64, ABI layout, distinct.  Allocates the
+ * scratch of dg_rhs_adjoint (six state-sized, one trace-sized buffer and one
+ * of n_f + 3 values per node, on the first use of either), and on its own
+ * first use traces, derived fields and rho_v of the three intermediate states
+ * if they take no more than a quarter of the device's free memory (see
+ * dg_set_adjoint_memory; without them each state is split a second time).
+ * DG_ENOTIMPL for float32 contexts (DG_FP32_BULK, DG_FP32_PERT); asynchronous. */
 int dg_adjoint_step(dg_ctx *ctx, double dt, const void *U_n, const double *lam_np1,
                     double *lam_n);
+
+/* Whether dg_adjoint_step may keep the traces, derived fields and rho_v of its
+ * intermediate states in the context (keep = 1, the default; the next
+ * dg_adjoint_step decides by the free memory then) or not (keep = 0: gives
+ * back what it holds, after synchronising the stream).  The results agree to
+ * rounding.  Errors: DG_EINVAL, DG_ENOTIMPL for float32 contexts, DG_ECUDA. */
+int dg_set_adjoint_memory(dg_ctx *ctx, int keep);
 
 /* Cloud-water functional J(U) = integral of rho_c = rho_m - rho_v over the
  * domain (Gauss rule of the DG space; rho_v from the split Eq. (2.8)) and

@@ -432,8 +432,7 @@ void release(dg_ctx *c) {
     void *ptrs[] = {c->U[0], c->U[1], c->derived, c->trace[0], c->trace[1], c->bnode_d,
                     c->bface_d, c->bnode_r, c->bface_r, c->flags, c->partials, c->rvs_tab,
                     c->adjX[0], c->adjX[1], c->adjX[2], c->adjL[0], c->adjL[1], c->adjL[2],
-                    c->ubar_part, c->tadj, c->adjRv[0], c->adjD[1], c->adjD[2], c->adjD[3],
-                    c->adjT[1], c->adjT[2], c->adjT[3], c->adjRv[1], c->adjRv[2], c->adjRv[3], c->bsplit, c->fbuf, c->ftab, c->alphaK, c->alphaV,
+                    c->ubar_part, c->tadj, c->adj_sets, c->bsplit, c->fbuf, c->ftab, c->alphaK, c->alphaV,
                     c->dtrace[0], c->dtrace[1], c->sponge, c->fallout};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -541,55 +540,83 @@ int upload_base(dg_ctx *c, const double *node_tab, const double *face_tab) {
     return DG_OK;
 }
 
-// Scratch of the adjoint entry points, on first use.  Set 0 (derived fields,
-// rho_v and traces of one state) uses the context's own buffers.  A reversed
-// step keeps the sets of all four stage states, so that none is split twice
-// (four of five k_prepare launches less; the adjoint step of 128x64 order 4:
-// 1.65 -> 1.51 ms); where the device has no room for the other three it does
-// with set 0 and splits each state again.
+// Scratch of the adjoint entry points, on first use
 int ensure_adjoint(dg_ctx *c) {
     if (c->ubar_part) return DG_OK;
     const size_t state = (size_t)c->nodes * c->nf * sizeof(double);
     const size_t trace = (size_t)2 * c->cfg.dim * c->ne * c->trace_face * sizeof(double);
-    const size_t derived = (size_t)c->nodes * c->nd * sizeof(double), rv = (size_t)c->nodes * sizeof(double);
     int st = DG_OK;
-    c->adjD[0] = (double *)c->derived;
-    c->adjT[0] = (double *)c->trace[0];
-    if (!c->adjRv[0]) st = alloc(c, (void **)&c->adjRv[0], rv);
     for (int i = 0; i < 3 && st == DG_OK; ++i)
         if (!c->adjX[i]) st = alloc(c, &c->adjX[i], state);
     for (int i = 0; i < 3 && st == DG_OK; ++i)
         if (!c->adjL[i]) st = alloc(c, (void **)&c->adjL[i], state);
     if (st == DG_OK && !c->tadj) st = alloc(c, (void **)&c->tadj, trace);
     if (st == DG_OK) st = alloc(c, (void **)&c->ubar_part, (size_t)c->nodes * c->ntr * sizeof(double));
-    if (st != DG_OK) return st;
-    for (int k = 1; k < 4 && st == DG_OK; ++k) {
-        st = alloc(c, (void **)&c->adjD[k], derived);
-        if (st == DG_OK) st = alloc(c, (void **)&c->adjT[k], trace);
-        if (st == DG_OK) st = alloc(c, (void **)&c->adjRv[k], rv);
-    }
-    if (st != DG_OK) {
-        for (int k = 1; k < 4; ++k) {
-            c->device_bytes -= (c->adjD[k] ? derived : 0) + (c->adjT[k] ? trace : 0) + (c->adjRv[k] ? rv : 0);
-            for (double **p : {&c->adjD[k], &c->adjT[k], &c->adjRv[k]}) {
-                if (*p) cudaFree(*p);
-                *p = nullptr;
-            }
-        }
-    }
-    return DG_OK;
+    return st;
 }
 
-// split and traces of U with rho_v, for the adjoint kernels, into set k (rho_v
-// into `rv` if given: derive_and_store writes it after 1/rho, so it may take
-// the place of 1/rho, which the adjoint kernels do not read)
-int prepare_adjoint(dg_ctx *c, const void *U, int k, double *rv = nullptr) {
+void drop_adjoint_sets(dg_ctx *c) {
+    if (!c->adj_sets) return;
+    cudaFree(c->adj_sets);
+    c->adj_sets = nullptr;
+    c->device_bytes -= c->adj_sets_bytes;
+}
+
+// The sets of a reversed step (derived fields, rho_v and traces of its four
+// stage states), so that none is split twice: four of five k_prepare launches
+// less, the adjoint step of 128x64 order 4 1.65 -> 1.51 ms.  Set 0 has the
+// context's own derived fields and traces.  Made by the first reversed step in
+// one allocation, and only where it takes at most a quarter of the device's
+// free memory: it is an option, and the rest is the caller's.  Without the
+// sets each state is split again, with the same result.
+bool have_adjoint_sets(dg_ctx *c) {
+    if (c->adj_sets || c->adj_sets_off) return c->adj_sets != nullptr;
+    c->adj_sets_off = true;     // decided once
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t trace = up((size_t)2 * c->cfg.dim * c->ne * c->trace_face * sizeof(double));
+    const size_t derived = up((size_t)c->nodes * c->nd * sizeof(double));
+    const size_t rv = up((size_t)c->nodes * sizeof(double));
+    c->adj_sets_bytes = 3 * (trace + derived) + 4 * rv;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (c->adj_sets_bytes > free_bytes / 4) return false;
+    if (alloc(c, &c->adj_sets, c->adj_sets_bytes) != DG_OK) return false;
+    char *p = (char *)c->adj_sets;
+    auto take = [&p](size_t b) { p += b; return (double *)(p - b); };
+    for (int k = 0; k < 4; ++k) {
+        c->adjD[k] = k ? take(derived) : (double *)c->derived;
+        c->adjT[k] = k ? take(trace) : (double *)c->trace[0];
+        c->adjRv[k] = take(rv);
+    }
+    return true;
+}
+
+// Derived fields, rho_v and traces of a state, as the adjoint kernels read them
+struct AdjSet {
+    double *derived, *rv, *trace;
+};
+
+AdjSet adj_set(const dg_ctx *c, int k) { return {c->adjD[k], c->adjRv[k], c->adjT[k]}; }
+
+// In the context's own buffers: rho_v takes the place of 1/rho, which the
+// adjoint kernels do not read (derive_and_store writes it after 1/rho); a
+// stage does read 1/rho, so this set serves no stage.
+AdjSet own_adj_set(const dg_ctx *c) {
+    double *d = (double *)c->derived;
+    return {d, d + c->nodes, (double *)c->trace[0]};
+}
+
+// split and traces of U with rho_v, for the adjoint kernels
+int prepare_adjoint(dg_ctx *c, const void *U, const AdjSet &s) {
     c->derived_valid = false;
     KArgs<double> A = base_args<double>(c, c->ref64);
     A.Uin = (const double *)U;
-    A.derived_out = c->adjD[k];
-    A.rv_out = rv ? rv : c->adjRv[k];
-    A.trace_out = c->adjT[k];
+    A.derived_out = s.derived;
+    A.rv_out = s.rv;
+    A.trace_out = s.trace;
     return cuda_status(c->L64->prepare(A, false, c->stream));
 }
 
@@ -616,16 +643,16 @@ int stage_adjoint(dg_ctx *c, const void *Uin, const void *Un, void *Uout, int k,
     return st;
 }
 
-AdjArgs adj_args(const dg_ctx *c, const void *U, int k, const double *w, double *out, double alpha,
-                 double beta, double gamma) {
+AdjArgs adj_args(const dg_ctx *c, const void *U, const AdjSet &s, const double *w, double *out,
+                 double alpha, double beta, double gamma) {
     AdjArgs A;
     std::memset(&A, 0, sizeof(A));
     A.M = c->M;
     A.ref = c->ref64;
     A.U = (const double *)U;
-    A.derived = c->adjD[k];
-    A.rv = c->adjRv[k];
-    A.trace = c->adjT[k];
+    A.derived = s.derived;
+    A.rv = s.rv;
+    A.trace = s.trace;
     A.bnode = c->bnode_d;
     A.bface = c->bface_d;
     A.rvs_tab = c->rvs_tab;
@@ -640,10 +667,10 @@ AdjArgs adj_args(const dg_ctx *c, const void *U, int k, const double *w, double 
 }
 
 // out = alpha out + beta w + gamma (dR/dU (U))^T w, the split and traces of U
-// in set k
-int rhs_adjoint_into(dg_ctx *c, const void *U, int k, const double *w, double *out, double alpha,
+// in set s
+int rhs_adjoint_into(dg_ctx *c, const void *U, const AdjSet &s, const double *w, double *out, double alpha,
                      double beta, double gamma) {
-    AdjArgs A = adj_args(c, U, k, w, out, alpha, beta, gamma);
+    AdjArgs A = adj_args(c, U, s, w, out, alpha, beta, gamma);
     if (c->LA->local(A, c->stream) != cudaSuccess) return DG_ECUDA;
     if (c->LA->gather(A, c->stream) != cudaSuccess) return DG_ECUDA;
     return DG_OK;
@@ -1181,9 +1208,10 @@ int dg_rhs_adjoint(dg_ctx *c, const void *U, const double *w, double *ubar) {
     DeviceGuard dg(c->device);
     int st = ensure_adjoint(c);
     if (st != DG_OK) return st;
-    st = prepare_adjoint(c, U, 0);
+    const AdjSet s = own_adj_set(c);
+    st = prepare_adjoint(c, U, s);
     if (st != DG_OK) return st;
-    return rhs_adjoint_into(c, U, 0, w, ubar, 0.0, 0.0, 1.0);
+    return rhs_adjoint_into(c, U, s, w, ubar, 0.0, 0.0, 1.0);
 }
 
 int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1, double *lam_n) {
@@ -1199,9 +1227,9 @@ int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1
     //   U1 = U^n + dt/2 R(U^n); U2 = U1 + dt/2 R(U1); U3 = 2/3 U^n + 1/3 U2 + dt/6 R(U2)
     void *X1 = c->adjX[0], *X2 = c->adjX[1], *X3 = c->adjX[2];
     const void *X[4] = {U_n, X1, X2, X3};
-    const bool sets = c->adjRv[3] != nullptr;    // every stage state's split and traces kept
+    const bool sets = have_adjoint_sets(c);    // every stage state's split and traces kept
     if (sets) {
-        st = prepare_adjoint(c, U_n, 0);
+        st = prepare_adjoint(c, U_n, adj_set(c, 0));
         if (st == DG_OK) st = stage_adjoint(c, U_n, U_n, X1, 0, 0.0, 1.0, 0.5 * dt);
         if (st == DG_OK) st = stage_adjoint(c, X1, X1, X2, 1, 0.0, 1.0, 0.5 * dt);
         if (st == DG_OK) st = stage_adjoint(c, X2, U_n, X3, 2, 2.0 / 3.0, 1.0 / 3.0, dt / 6.0);
@@ -1214,8 +1242,9 @@ int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1
     if (st != DG_OK) return st;
     // out = alpha out + beta w + gamma (dR/dU (X_k))^T w
     auto reverse = [&](int k, const double *w, double *out, double alpha, double beta, double gamma) {
-        const int p = sets ? DG_OK : prepare_adjoint(c, X[k], 0);
-        return p != DG_OK ? p : rhs_adjoint_into(c, X[k], sets ? k : 0, w, out, alpha, beta, gamma);
+        const AdjSet s = sets ? adj_set(c, k) : own_adj_set(c);
+        const int p = sets ? DG_OK : prepare_adjoint(c, X[k], s);
+        return p != DG_OK ? p : rhs_adjoint_into(c, X[k], s, w, out, alpha, beta, gamma);
     };
     // reverse: U^{n+1} = U3 + dt/2 R(U3)
     double *l3 = c->adjL[0], *l2 = c->adjL[1], *l1 = c->adjL[2];
@@ -1230,20 +1259,29 @@ int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1
     return reverse(0, l1, lam_n, 2.0 / 3.0, 1.0, 0.5 * dt);
 }
 
+int dg_set_adjoint_memory(dg_ctx *c, int keep) {
+    if (!c || (keep != 0 && keep != 1)) return DG_EINVAL;
+    if (c->fp32 || !c->LA) return DG_ENOTIMPL;
+    DeviceGuard dg(c->device);
+    if (!keep) {
+        if (c->adj_sets && cudaStreamSynchronize(c->stream) != cudaSuccess) return DG_ECUDA;
+        drop_adjoint_sets(c);
+    }
+    c->adj_sets_off = !keep;
+    return DG_OK;
+}
+
 int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     if (!c || !U || !J || !dJdU || (const void *)dJdU == U) return DG_EINVAL;
     if (c->fp32 || !c->LA) return DG_ENOTIMPL;
     if (!c->base_set) return DG_ESTATE;
     DeviceGuard dg(c->device);
-    c->adjD[0] = (double *)c->derived;
-    c->adjT[0] = (double *)c->trace[0];
-    // rho_v in the place of 1/rho: dJdU may be U itself (k_cloud reads a node's
-    // state before it writes that node's gradient), so nothing passes through it
-    double *rv = c->adjD[0] + c->nodes;
-    const int st = prepare_adjoint(c, U, 0, rv);
+    // dJdU may be U itself: k_cloud reads a node's state before it writes that
+    // node's gradient, and rho_v stands in the derived fields
+    const AdjSet s = own_adj_set(c);
+    const int st = prepare_adjoint(c, U, s);
     if (st != DG_OK) return st;
-    AdjArgs A = adj_args(c, U, 0, nullptr, dJdU, 0.0, 0.0, 1.0);
-    A.rv = rv;
+    AdjArgs A = adj_args(c, U, s, nullptr, dJdU, 0.0, 0.0, 1.0);
     if (c->LA->cloud(A, c->partials, c->nred, c->stream) != cudaSuccess) return DG_ECUDA;
     std::vector<double> h(c->nred);
     if (cudaMemcpyAsync(h.data(), c->partials, sizeof(double) * c->nred, cudaMemcpyDeviceToHost,

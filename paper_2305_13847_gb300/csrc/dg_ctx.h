@@ -53,7 +53,11 @@ struct dg_ctx {
     double *adjL[3] = {nullptr, nullptr, nullptr};
     double *ubar_part = nullptr, *tadj = nullptr;
     // derived fields, rho_v and traces of the stage states of a reversed step
-    // (0: of U^n; all or none of 1 .. 3: see ensure_adjoint)
+    // (0: of U^n), in one allocation (have_adjoint_sets); off: none is wanted
+    // or none was to be had
+    void *adj_sets = nullptr;
+    size_t adj_sets_bytes = 0;
+    bool adj_sets_off = false;
     double *adjD[4] = {}, *adjT[4] = {}, *adjRv[4] = {};
     int nred = 0;
     std::vector<double> z_node, z_face;

@@ -101,6 +101,7 @@ SIGNATURES = [
     ("dg_rhs_noalloc", _I, [ctypes.POINTER(dg_config), _VP, _VP, _VP, _VP, _VP]),
     ("dg_rhs_noalloc_status", _I, [_VP, _VP]),
     ("dg_rhs_adjoint", _I, [_VP, _VP, _VP, _VP]),
+    ("dg_set_adjoint_memory", _I, [_VP, _I]),
     ("dg_cloud_functional", _I, [_VP, _VP, ctypes.POINTER(ctypes.c_double), _VP]),
     ("dg_set_stabilisation", _I, [_VP, ctypes.POINTER(dg_stabilisation)]),
     ("dg_ensemble_create", _I, [ctypes.POINTER(_VP), _I, _VP, _VP, _VP]),
@@ -291,6 +292,11 @@ def dg_adjoint_step_status(ctx, dt, U_n, lam_np1, lam_n):
 
 def dg_rhs_adjoint(ctx, U, w, ubar):
     _check(lib().dg_rhs_adjoint(ctx, _addr(U), _addr(w), _addr(ubar)), "dg_rhs_adjoint")
+
+
+def dg_set_adjoint_memory(ctx, keep):
+    """Whether dg_adjoint_step may keep its intermediate states' split and traces in the context."""
+    _check(lib().dg_set_adjoint_memory(ctx, int(keep)), "dg_set_adjoint_memory")
 
 
 def dg_cloud_functional(ctx, U, dJdU):

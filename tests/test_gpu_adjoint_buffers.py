@@ -28,3 +28,43 @@ def test_cloud_functional_in_place(dim, n, order):
         assert np.array_equal(V.cpu().numpy(), g.cpu().numpy())
     finally:
         dm.dg_free(ctx)
+
+
+def _scratch(prob):
+    """Bytes of dg_rhs_adjoint's scratch: six states, the traces and n_f + 3 values per node."""
+    mesh = prob.mesh
+    nodes, ntr = mesh.Ne * (mesh.k + 1) ** mesh.dim, prob.nf + 3
+    trace = 2 * mesh.dim * mesh.Ne * (mesh.k + 1) ** (mesh.dim - 1) * ntr
+    return 8 * (6 * prob.nf * nodes + trace + ntr * nodes)
+
+
+@pytest.mark.parametrize("dim,n,order", [(2, (7, 5), 3), (3, (3, 2, 3), 4)])
+def test_adjoint_step_with_and_without_kept_states(dim, n, order):
+    """Only dg_adjoint_step holds the intermediate states' split and traces, gives them back when told
+    to, and without them returns the same adjoint: within 1e-12 of each field's norm, twelve times the
+    8e-14 that either lies off the adjoint in exact arithmetic (the split's rounding is all that differs)."""
+    prob = _problem(dim, n, order)
+    U = to_device(perturbed_state(prob, seed=43), torch.float64)
+    g = torch.Generator().manual_seed(7)
+    lam = torch.randn(U.shape, generator=g, dtype=torch.float64).cuda()
+    ctx = library_context(prob)
+    try:
+        held = dm.dg_get_info(ctx).device_bytes
+        out = [torch.empty_like(U) for _ in range(4)]
+        dm.dg_rhs_adjoint(ctx, U, lam, out[3])
+        assert dm.dg_get_info(ctx).device_bytes - held == _scratch(prob)
+        held += _scratch(prob)
+        dm.dg_set_adjoint_memory(ctx, 0)
+        dm.dg_adjoint_step(ctx, 0.02, U, lam, out[0])
+        assert dm.dg_get_info(ctx).device_bytes == held
+        dm.dg_set_adjoint_memory(ctx, 1)
+        dm.dg_adjoint_step(ctx, 0.02, U, lam, out[1])
+        assert dm.dg_get_info(ctx).device_bytes > held
+        dm.dg_set_adjoint_memory(ctx, 0)
+        assert dm.dg_get_info(ctx).device_bytes == held
+        dm.dg_adjoint_step(ctx, 0.02, U, lam, out[2])
+        a, b, c = (o.cpu().numpy().reshape(prob.nf, -1) for o in out[:3])
+    finally:
+        dm.dg_free(ctx)
+    assert np.array_equal(a, c)
+    assert np.all(np.linalg.norm(a - b, axis=1) <= 1e-12 * np.linalg.norm(a, axis=1))
