@@ -7,6 +7,7 @@
 
 #include "dg_column.cuh"
 #include "dg_device.cuh"
+#include "dg_once.h"
 #include "dg_stage64.cuh"
 
 namespace dgm {
@@ -64,6 +65,19 @@ inline cudaError_t launch(K kern, int grid, int block, size_t smem, cudaStream_t
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Opt-in of a kernel to its dynamic shared memory on the current device (the
+// attribute is the device's own: several tiles need more than the default
+// 48 KB, and a context may be on any device)
+template <class K>
+inline cudaError_t allow_smem(OncePerDevice &once, K kern, size_t smem) {
+    int dev = 0;
+    const cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    return (cudaError_t)once(dev, [&] {
+        return (int)cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    });
+}
+
 template <class S, typename Real>
 struct Impl {
     static constexpr bool F64 = std::is_same<Real, double>::value;
@@ -92,13 +106,9 @@ struct Impl {
     static cudaError_t launch_prepare(const KArgs<Real> &A, cudaStream_t st) {
         constexpr size_t smem = prep_smem<DIFF>();
         const auto kern = prepare_kernel<DIFF>();
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t err =
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (err != cudaSuccess) return err;
-            attr = true;
-        }
+        static OncePerDevice once;
+        const cudaError_t err = allow_smem(once, kern, smem);
+        if (err != cudaSuccess) return err;
         return launch(kern, A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st, true, A);
     }
 
@@ -122,13 +132,9 @@ struct Impl {
     static cudaError_t launch_stage(const KArgs<Real> &A, cudaStream_t st) {
         constexpr size_t smem = stage_smem<PF, DIFF>();
         const auto kern = stage_kernel<MODE, PF, DIFF>();
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t err =
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (err != cudaSuccess) return err;
-            attr = true;
-        }
+        static OncePerDevice once;
+        const cudaError_t err = allow_smem(once, kern, smem);
+        if (err != cudaSuccess) return err;
         return launch(kern, A.ntiles > 0 ? A.ntiles : blocks(A), S::NT, smem, st, !PF, A);
     }
 
@@ -179,13 +185,9 @@ struct Impl {
     static cudaError_t launch_column(const KArgs<Real> &A, cudaStream_t st) {
         using C = ColShape<S>;
         constexpr size_t smem = column_smem_bytes<S, Real>();
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t err = cudaFuncSetAttribute(k_column<S, Real, MODE>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (err != cudaSuccess) return err;
-            attr = true;
-        }
+        static OncePerDevice once;
+        const cudaError_t err = allow_smem(once, &k_column<S, Real, MODE>, smem);
+        if (err != cudaSuccess) return err;
         const int nxb = (A.M.n[0] + C::BX - 1) / C::BX;
         const int nyb = S::D == 3 ? (A.M.n[1] + C::BY - 1) / C::BY : 1;
         k_column<S, Real, MODE><<<nxb * nyb, C::NT, smem, st>>>(A);
@@ -274,13 +276,9 @@ template <class S>
 struct AdjImpl {
     static constexpr size_t smem = adj_smem_bytes<S>();
     static cudaError_t local(const AdjArgs &A, cudaStream_t st) {
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t err = cudaFuncSetAttribute(k_adj_local<S>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (err != cudaSuccess) return err;
-            attr = true;
-        }
+        static OncePerDevice once;
+        const cudaError_t err = allow_smem(once, &k_adj_local<S>, smem);
+        if (err != cudaSuccess) return err;
         k_adj_local<S><<<(A.M.ne + S::EPB - 1) / S::EPB, S::NT, smem, st>>>(A);
         return cudaGetLastError();
     }
