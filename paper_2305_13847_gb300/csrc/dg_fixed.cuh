@@ -21,6 +21,9 @@
 // Groups whose E lies outside [kFxMinE, kFxMaxE] are the caller's business:
 // below, the values are flushed to zero (2^-823); above (and for infinities
 // and NaN, whose biased exponent is 2047) the caller takes the float64 sums.
+// The absolute error is the group's, so one huge value costs its whole group
+// the bits below 2^-57 of it: the caller draws its own line (fx_group,
+// dg_stage64.cuh) well above any physical value and far below kFxMaxE.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -80,15 +80,30 @@ __device__ __forceinline__ void fx_coef_fill(const KArgs<double> &A, int2 *s_cf)
 // a per-direction exponent of the coefficient tables by a run-time direction
 __device__ __forceinline__ int pick3(const int *q, int j) { return j == 0 ? q[0] : (j == 1 ? q[1] : q[2]); }
 
-// group exponents of N groups from the CTA's maxima (clamped below); true if
-// any group leaves the fixed-point range (then every thread takes float64)
-template <int N>
-__device__ __forceinline__ bool fx_group(const int *s_e, int *E) {
+// Bits of the values of a group that are taken as fixed point, |x| < 2^bits:
+// densities, mass fluxes and temperatures (kg/m^3, kg/m^2/s, K) 2^14, momenta
+// with their fluxes and p' (Pa) 2^22, energies and energy fluxes (J/m^3, W/m^2)
+// 2^34 -- 30 to 60 times what air at 1 bar and the speed of sound has.  A tile
+// with a larger value in it takes float64 sums: the elements of a tile share
+// the scale, and one that blows up must not cost the others their bits.  Below
+// the line it costs them at most 2^-57 of it: 1e-13 kg/m^2/s, 3e-11 Pa,
+// 1e-7 W/m^2, the rounding of the base state's own p, E and rho.
+// k: a field, or S::NF, + 1, + 2 for T, rho_v, p'.
+template <class S>
+__host__ __device__ constexpr int fx_bits(int k) {
+    return k < S::IM || k == S::NF || k == S::NF + 1 ? 14 : (k == S::IE ? 34 : 22);
+}
+
+// group exponents of the first N of the fields and T, rho_v, p' from the CTA's
+// maxima (clamped below), with q of the coefficients in them; true if any
+// group leaves the fixed-point range (then every thread takes float64)
+template <class S, int N>
+__device__ __forceinline__ bool fx_group(const int *s_e, int q, int *E) {
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         E[k] = max(s_e[k], kFxMinE);
-        bad = bad || E[k] > kFxMaxE;
+        bad = bad || E[k] > min(kFxMaxE, 1022 + fx_bits<S>(k) + q);
     }
     return bad;
 }
@@ -145,7 +160,7 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
     for (int f = 0; f < S::NTR; ++f) E[f] = valid && fx_field<S>(f) ? fx_expo(v[f]) : 0;
     fx_reduce_max<S::NTR>(E, s_e + FxExp<S, DIFF>::TRACE);
     __syncthreads();
-    if (fx_group<S::NTR>(s_e + FxExp<S, DIFF>::TRACE, E)) {
+    if (fx_group<S, S::NTR>(s_e + FxExp<S, DIFF>::TRACE, 0, E)) {
         if (valid) {
 #pragma unroll
             for (int f = 0; f < S::NTR; ++f) s_tr[f * STR + t] = v[f];
@@ -455,7 +470,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
         __syncthreads();
         fx_reduce_max<S::NF>(E, s_e + X::NODE);
         __syncthreads();
-        const bool bad = fx_group<S::NF>(s_e + X::NODE, E);
+        const bool bad = fx_group<S, S::NF>(s_e + X::NODE, 0, E);
         if (valid) {
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
@@ -553,7 +568,10 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     // and the lift of the face fluxes, R_a -= (2/h_j) l_a(s)/w_a Fhat(j, s).
     // The low face holds the outward flux (inline) or G along +e_j, minus
     // this element's outward flux (face pass), hence the sign.
-    const bool bad = fx_group<S::NF>(s_e + X::FLUX, ex);
+    int q = A.ref.q_vol[0];
+#pragma unroll
+    for (int j = 0; j < S::D; ++j) q = max(q, max(A.ref.q_vol[j], A.ref.q_lift[j]));
+    const bool bad = fx_group<S, S::NF>(s_e + X::FLUX, q, ex);
     double R[S::NF];
     if (!bad) {
         // in place: each thread converts the words that it wrote or scanned
@@ -626,7 +644,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
             }
         }
     } else if (valid) {
-        // values outside the fixed-point range (infinities, NaN): float64 sums
+        // values outside the fixed-point range (blown up, infinite, NaN): float64 sums
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) R[f] = line_sums<S, PF, DIFF, FACE>(A, s_fl, s_fh, el, a, f);
     }
