@@ -642,7 +642,9 @@ __device__ __forceinline__ float rain_velocity(float rr, float rm, const MeshDat
     const float rrp = rr > 0.0f ? rr : 0.0f;
     const float rw = M.rho_w_f > 0.0f ? M.rho_w_f : rm + rr;
     if (!(rrp > 0.0f) || !(rw > 0.0f)) return 0.0f;
-    return M.kvr_f * exp2f(0.125f * __log2f(rrp * frcp(rw)));
+    // a trace of rain in dry air leaves rho_w subnormal: outside frcp's range, divided
+    const float t = (rw >= kFrcpMin && rw <= kFrcpMax) ? rrp * frcp(rw) : rrp / rw;
+    return M.kvr_f * exp2f(0.125f * __log2f(t));
 }
 
 // Per-node split plus the node-local quantities the next operator needs.

@@ -111,9 +111,13 @@ __device__ __forceinline__ double rsqrt_seed(double x) {
 
 // float32 1/x: the hardware's approximation (1 ulp) and one Newton step, three
 // instructions and within 0.51 ulp, where __frcp_rn is a dozen with a branch.
-// Zero and infinities give NaN (the callers' densities, temperatures and
-// Newton derivatives are neither in a physical state, and a state that is not
-// physical is counted by its own checks).
+// For kFrcpMin <= |x| <= kFrcpMax, where x and 1/x are normal: a subnormal x,
+// zero and infinities give NaN, a larger x 0.  (The densities, temperatures
+// and Newton derivatives that come here are of order 1e-3 to 1e9 in a physical
+// state, and a state that is not physical is counted by its own checks; where
+// the argument may be any positive number the caller checks the range.)
+constexpr float kFrcpMin = 0x1p-126f, kFrcpMax = 0x1p126f;
+
 __device__ __forceinline__ float frcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
