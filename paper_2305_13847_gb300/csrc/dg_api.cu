@@ -1276,8 +1276,6 @@ int dg_cloud_functional(dg_ctx *c, const void *U, double *J, double *dJdU) {
     if (c->fp32 || !c->LA) return DG_ENOTIMPL;
     if (!c->base_set) return DG_ESTATE;
     DeviceGuard dg(c->device);
-    // dJdU may be U itself: k_cloud reads a node's state before it writes that
-    // node's gradient, and rho_v stands in the derived fields
     const AdjSet s = own_adj_set(c);
     const int st = prepare_adjoint(c, U, s);
     if (st != DG_OK) return st;
