@@ -202,7 +202,7 @@ namespace dgm {
 // The float64 reference tables of order k with the volume derivative and
 // lift coefficients scaled by 2/h_j of a mesh: the tables every float64 stage
 // kernel takes (dg_init_mesh, dg_rhs_noalloc).
-RefData<double> scaled_ref64(int order, const double two_over_h[3]) {
+RefData<double> scaled_ref64(int dim, int order, const double two_over_h[3]) {
     RefData<double> r = make_ref<double>(order);
     for (int j = 0; j < 3; ++j)
         for (int a = 0; a < 6; ++a) {
@@ -234,6 +234,8 @@ RefData<double> scaled_ref64(int order, const double two_over_h[3]) {
         r.q_dtrace[j] = above(dt, 12);
     }
     r.q_trace = above(r.lp, 6, above(r.lm, 6));
+    r.q_max = r.q_vol[0];
+    for (int j = 0; j < dim; ++j) r.q_max = std::max(r.q_max, std::max(r.q_vol[j], r.q_lift[j]));
     return r;
 }
 }  // namespace dgm
@@ -788,7 +790,7 @@ int dg_init_mesh(dg_ctx **out, const dg_config *cfg, void *cuda_stream) {
     mesh_float_copies(M);
     // the volume derivative and lift tables pre-scaled by 2/h_j of this
     // mesh, float64 and their float32 roundings
-    c->ref64 = scaled_ref64(g.order, M.two_over_h);
+    c->ref64 = scaled_ref64(g.dim, g.order, M.two_over_h);
     c->ref32 = make_ref<float>(g.order);
     for (int j = 0; j < 3; ++j)
         for (int a = 0; a < 6; ++a) {

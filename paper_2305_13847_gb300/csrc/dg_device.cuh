@@ -129,8 +129,9 @@ struct RefData {
     Real liftm_s[3][6], liftp_s[3][6];    // (2/h_j) l_a(-+1)/w_a
     Real dliftm_s[3][6], dliftp_s[3][6];  // (2/h_j)^2 l_a'(-+1)/w_a
     // float64 tables: |entry| < 2^q for the scaled tables dhat_s, lift*_s, dlift*_s,
-    // (2/h_j) dmat, (2/h_j) dl* and for l* (fixed-point contractions, dg_fixed.cuh)
-    int q_vol[3], q_lift[3], q_dlift[3], q_dmat[3], q_dtrace[3], q_trace;
+    // (2/h_j) dmat, (2/h_j) dl* and for l* (fixed-point contractions, dg_fixed.cuh);
+    // q_max: the largest of q_vol and q_lift over the mesh's directions
+    int q_vol[3], q_lift[3], q_dlift[3], q_dmat[3], q_dtrace[3], q_trace, q_max;
 };
 
 template <typename Real>

@@ -22,7 +22,7 @@
 // below, the values are flushed to zero (2^-823); above (and for infinities
 // and NaN, whose biased exponent is 2047) the caller takes the float64 sums.
 // The absolute error is the group's, so one huge value costs its whole group
-// the bits below 2^-57 of it: the caller draws its own line (fx_group,
+// the bits below 2^-57 of it: the caller draws its own line (fx_limit,
 // dg_stage64.cuh) well above any physical value and far below kFxMaxE.
 #pragma once
 
@@ -32,6 +32,7 @@ namespace dgm {
 
 constexpr int kFxMinE = 200;
 constexpr int kFxMaxE = 1900;
+constexpr int kFxOutE = 4095;    // marks a group as out of range
 
 // biased exponent of x (0 for zero and subnormals, 2047 for infinities and NaN)
 __device__ __forceinline__ int fx_expo(double x) {
@@ -94,9 +95,10 @@ __device__ __forceinline__ long long fx_shift(long long v, int d) {
 
 // s_e[k] = max(s_e[k], e[k] over the CTA) for N <= 32 groups: one warp
 // reduction per group, then one shared-memory atomic per warp with a group
-// per lane.  Called by whole warps.
+// per lane, which enters a group above its limit as out of range.  limit: that
+// of group threadIdx.x % 32.  Called by whole warps.
 template <int N>
-__device__ __forceinline__ void fx_reduce_max(const int *e, int *s_e) {
+__device__ __forceinline__ void fx_reduce_max(const int *e, int limit, int *s_e) {
     const int lane = threadIdx.x & 31;
     int mine = 0;
 #pragma unroll
@@ -104,6 +106,7 @@ __device__ __forceinline__ void fx_reduce_max(const int *e, int *s_e) {
         const int r = __reduce_max_sync(0xffffffffu, e[k]);
         if (lane == k) mine = r;
     }
+    if (mine > limit) mine = kFxOutE;
     if (lane < N && mine > 0) atomicMax(s_e + lane, mine);
 }
 

@@ -229,7 +229,7 @@ const Launchers<double> *launchers_d3_f64(int K, int rain);
 const Launchers<float> *launchers_d2_f32(int K, int rain);
 const Launchers<float> *launchers_d3_f32(int K, int rain);
 // float64 reference tables with the coefficients scaled by 2/h_j (dg_api.cu)
-RefData<double> scaled_ref64(int order, const double two_over_h[3]);
+RefData<double> scaled_ref64(int dim, int order, const double two_over_h[3]);
 
 }  // namespace dgm
 

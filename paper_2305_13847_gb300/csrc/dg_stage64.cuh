@@ -88,22 +88,24 @@ __device__ __forceinline__ int pick3(const int *q, int j) { return j == 0 ? q[0]
 // the scale, and one that blows up must not cost the others their bits.  Below
 // the line it costs them at most 2^-57 of it: 1e-13 kg/m^2/s, 3e-11 Pa,
 // 1e-7 W/m^2, the rounding of the base state's own p, E and rho.
-// k: a field, or S::NF, + 1, + 2 for T, rho_v, p'.
+// Returns the largest exponent of group k (a field, or S::NF, + 1, + 2 for T,
+// rho_v, p') with coefficients below 2^q in it.  Evaluated by one lane per group
+// (fx_reduce_max): by every thread for every group it cost a small mesh 2 %.
 template <class S>
-__host__ __device__ constexpr int fx_bits(int k) {
-    return k < S::IM || k == S::NF || k == S::NF + 1 ? 14 : (k == S::IE ? 34 : 22);
+__device__ __forceinline__ int fx_limit(int k, int q) {
+    const int bits = k < S::IM || k == S::NF || k == S::NF + 1 ? 14 : (k == S::IE ? 34 : 22);
+    return min(kFxMaxE, 1022 + bits + q);
 }
 
-// group exponents of the first N of the fields and T, rho_v, p' from the CTA's
-// maxima (clamped below), with q of the coefficients in them; true if any
-// group leaves the fixed-point range (then every thread takes float64)
-template <class S, int N>
-__device__ __forceinline__ bool fx_group(const int *s_e, int q, int *E) {
+// group exponents of N groups from the CTA's maxima (clamped below); true if
+// any group leaves the fixed-point range (then every thread takes float64)
+template <int N>
+__device__ __forceinline__ bool fx_group(const int *s_e, int *E) {
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         E[k] = max(s_e[k], kFxMinE);
-        bad = bad || E[k] > min(kFxMaxE, 1022 + fx_bits<S>(k) + q);
+        bad = bad || E[k] > kFxMaxE;
     }
     return bad;
 }
@@ -158,9 +160,9 @@ __device__ __forceinline__ void write_traces64(const KArgs<double> &A, const dou
     int E[S::NTR];
 #pragma unroll
     for (int f = 0; f < S::NTR; ++f) E[f] = valid && fx_field<S>(f) ? fx_expo(v[f]) : 0;
-    fx_reduce_max<S::NTR>(E, s_e + FxExp<S, DIFF>::TRACE);
+    fx_reduce_max<S::NTR>(E, fx_limit<S>(t & 31, 0), s_e + FxExp<S, DIFF>::TRACE);
     __syncthreads();
-    if (fx_group<S, S::NTR>(s_e + FxExp<S, DIFF>::TRACE, 0, E)) {
+    if (fx_group<S::NTR>(s_e + FxExp<S, DIFF>::TRACE, E)) {
         if (valid) {
 #pragma unroll
             for (int f = 0; f < S::NTR; ++f) s_tr[f * STR + t] = v[f];
@@ -468,9 +470,9 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
 #pragma unroll
         for (int f = 0; f < S::NF; ++f) E[f] = valid && fx_field<S>(f) ? fx_expo(u[f]) : 0;
         __syncthreads();
-        fx_reduce_max<S::NF>(E, s_e + X::NODE);
+        fx_reduce_max<S::NF>(E, fx_limit<S>(t & 31, 0), s_e + X::NODE);
         __syncthreads();
-        const bool bad = fx_group<S, S::NF>(s_e + X::NODE, 0, E);
+        const bool bad = fx_group<S::NF>(s_e + X::NODE, E);
         if (valid) {
 #pragma unroll
             for (int f = 0; f < S::NF; ++f) {
@@ -560,7 +562,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
                 if (fx_field<S>(f)) ex[f] = max(ex[f], fx_expo(g[(S::NF + f) * S::NFP1]) + qd);
         }
     }
-    fx_reduce_max<S::NF>(ex, s_e + X::FLUX);
+    fx_reduce_max<S::NF>(ex, fx_limit<S>(t & 31, A.ref.q_max), s_e + X::FLUX);
     __syncthreads();
 
     // ---- phase 3: volume term of Eq. (3.2), sum factorised,
@@ -568,10 +570,7 @@ __device__ __forceinline__ void stage_block64(const KArgs<double> &A, int bidx, 
     // and the lift of the face fluxes, R_a -= (2/h_j) l_a(s)/w_a Fhat(j, s).
     // The low face holds the outward flux (inline) or G along +e_j, minus
     // this element's outward flux (face pass), hence the sign.
-    int q = A.ref.q_vol[0];
-#pragma unroll
-    for (int j = 0; j < S::D; ++j) q = max(q, max(A.ref.q_vol[j], A.ref.q_lift[j]));
-    const bool bad = fx_group<S, S::NF>(s_e + X::FLUX, q, ex);
+    const bool bad = fx_group<S::NF>(s_e + X::FLUX, ex);
     double R[S::NF];
     if (!bad) {
         // in place: each thread converts the words that it wrote or scanned

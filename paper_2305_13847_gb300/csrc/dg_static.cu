@@ -129,7 +129,7 @@ extern "C" int dg_rhs_noalloc(const dg_config *cfg, const double *base_node, con
     for (int j = 0; j < g.dim; ++j) M.jac *= M.h[j] / 2.0;
     M.newton_cap = kMaxNewton;
     // the reference tables of dg_init_mesh (scaled by 2/h_j of this mesh)
-    A.ref = scaled_ref64(g.order, M.two_over_h);
+    A.ref = scaled_ref64(g.dim, g.order, M.two_over_h);
 
     A.rvs_tab = reinterpret_cast<const double *>(scratch);
     A.flags = reinterpret_cast<unsigned long long *>(scratch + kTableBytes);
