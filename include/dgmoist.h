@@ -481,7 +481,11 @@ void dg_ensemble_free(dg_ensemble *ens);
  *                  isfinite(x), max(|x|, 1.5) against those of the library's
  *                  bit-pattern compares;
  *                  FF_SPLIT writes hi + lo of the float32 pair of x (in
- *                  float64) and, beside it, x itself;
+ *                  float64) and, beside it, x itself; RECIP_F32, RSQRT_F32,
+ *                  LOG1P_F32 and EXPM1_F32 take the float32-rounded x and
+ *                  stand beside the float64 function of it; FIXED writes the
+ *                  fixed-point value of x in a group whose exponent is i mod
+ *                  64 above that of x[i], beside x itself;
  *   out[2n .. 4n)  for FF_SPLIT the pair's hi and CUDA's float32 rounding
  *                  of x; for RHO_VS / RHO_VS_F32 / RHO_VS_BULK the derivative
  *                  d rho_vs / dT, the library's (RHO_VS_BULK: the float32
@@ -501,6 +505,11 @@ void dg_ensemble_free(dg_ensemble *ens);
 #define DG_MATH_COMPARE 9
 #define DG_MATH_RHO_VS_BULK 10
 #define DG_MATH_FF_SPLIT 11
+#define DG_MATH_RECIP_F32 12
+#define DG_MATH_RSQRT_F32 13
+#define DG_MATH_LOG1P_F32 14
+#define DG_MATH_EXPM1_F32 15
+#define DG_MATH_FIXED 16
 int dg_selftest_math(dg_ctx *ctx, int fn, const double *x, double *out, long long n);
 
 /* Float64 FMA throughput probe (a measurement aid, not part of the method):

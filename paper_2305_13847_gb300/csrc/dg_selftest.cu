@@ -4,10 +4,11 @@
 // The float64 kernels avoid CUDA's conversions, divisions, square roots and
 // pow on their hot paths (GB300 issues conversions and float64 compares to
 // the same slow pipe as the float64 arithmetic): narrow / widen are integer
-// operations on the bit pattern, recip / rsqrt_nr / sqrt_nr refine the
-// hardware's approximate reciprocal (square root) by Newton-Raphson steps,
-// inv_root16 / inv_root8 take one third-order step from a float32 estimate,
-// and rho_vs comes from a table of Taylor coefficients.  This entry point
+// operations on the bit pattern, recip / rsqrt_nr / sqrt_nr take one
+// third-order step from the hardware's approximate reciprocal (square root),
+// inv_root16 / inv_root8 one from a float32 estimate, rho_vs comes from a
+// table of Taylor coefficients, and the contractions are fixed point; the
+// float32 kernels have their own reciprocals, log1p and expm1.  This entry point
 // evaluates each of them and, beside it, the function it stands in for --
 // the hardware conversion, IEEE division and square root, CUDA's pow, the
 // closed form of Eq. (2.6) -- so that a test can hold them to their bounds.
@@ -94,6 +95,30 @@ __global__ void k_selftest_math(int fn, const double *__restrict__ x, double *__
                 ref2 = (double)__double2float_rn(v);
                 break;
             }
+            case DG_MATH_RECIP_F32:
+            case DG_MATH_RSQRT_F32:
+            case DG_MATH_LOG1P_F32:
+            case DG_MATH_EXPM1_F32: {
+                const float f = __double2float_rn(v);
+                const double d = (double)f;
+                ours = (double)(fn == DG_MATH_RECIP_F32   ? frcp(f)
+                                : fn == DG_MATH_RSQRT_F32 ? rsqrt_nr(f)
+                                : fn == DG_MATH_LOG1P_F32 ? log1p_small(f)
+                                                          : expm1_small(f));
+                ref = fn == DG_MATH_RECIP_F32   ? 1.0 / d
+                      : fn == DG_MATH_RSQRT_F32 ? 1.0 / sqrt(d)
+                      : fn == DG_MATH_LOG1P_F32 ? log1p(d)
+                                                : expm1(d);
+                break;
+            }
+            case DG_MATH_FIXED: {
+                // x = (h 2^28 + l) 2^(E - 1079), in fx_round's units of 2^(E - 1080)
+                const int E = max(fx_expo(v), kFxMinE) + (int)(i & 63);
+                const int2 w = fx_from(v, E);
+                ours = fx_round(2 * (((long long)w.x << 28) + w.y), E);
+                ref = v;
+                break;
+            }
             default: {
                 // DG_MATH_COMPARE: the bit-pattern compares against the
                 // constant 1.5 and zero; bit k of ours / ref is compare k
@@ -118,7 +143,7 @@ __global__ void k_selftest_math(int fn, const double *__restrict__ x, double *__
 }  // namespace
 
 extern "C" int dg_selftest_math(dg_ctx *c, int fn, const double *x, double *out, long long n) {
-    if (!c || !x || !out || n < 1 || fn < DG_MATH_NARROW || fn > DG_MATH_FF_SPLIT) return DG_EINVAL;
+    if (!c || !x || !out || n < 1 || fn < DG_MATH_NARROW || fn > DG_MATH_FIXED) return DG_EINVAL;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != c->device) return DG_EINVAL;
     const long long blocks = (n + 255) / 256;
