@@ -341,6 +341,7 @@ int dg_rhs_adjoint(dg_ctx *ctx, const void *U, const double *w, double *ubar);
  * first use traces, derived fields and rho_v of the three intermediate states
  * if they take no more than a quarter of the device's free memory (see
  * dg_set_adjoint_memory; without them each state is split a second time).
+ * A failing node counts twice per stage state in dg_check_status either way.
  * DG_ENOTIMPL for float32 contexts (DG_FP32_BULK, DG_FP32_PERT); asynchronous. */
 int dg_adjoint_step(dg_ctx *ctx, double dt, const void *U_n, const double *lam_np1,
                     double *lam_n);

@@ -611,10 +611,13 @@ AdjSet own_adj_set(const dg_ctx *c) {
     return {d, d + c->nodes, (double *)c->trace[0]};
 }
 
-// split and traces of U with rho_v, for the adjoint kernels
-int prepare_adjoint(dg_ctx *c, const void *U, const AdjSet &s) {
+// split and traces of U with rho_v, for the adjoint kernels; kept: the one
+// split of a stage state, in the place of the stage's own and the reversal's,
+// so that a reversed step counts a failing node twice per state either way
+int prepare_adjoint(dg_ctx *c, const void *U, const AdjSet &s, bool kept = false) {
     c->derived_valid = false;
     KArgs<double> A = base_args<double>(c, c->ref64);
+    A.fail_extra = kept;
     A.Uin = (const double *)U;
     A.derived_out = s.derived;
     A.rv_out = s.rv;
@@ -627,6 +630,7 @@ int prepare_adjoint(dg_ctx *c, const void *U, const AdjSet &s) {
 int stage_adjoint(dg_ctx *c, const void *Uin, const void *Un, void *Uout, int k, double alpha, double beta,
                   double gdt) {
     KArgs<double> A = base_args<double>(c, c->ref64);
+    A.fail_extra = 1;     // see prepare_adjoint
     A.fallout = nullptr;
     A.Uin = (const double *)Uin;
     A.Un = (const double *)Un;
@@ -1231,7 +1235,7 @@ int dg_adjoint_step(dg_ctx *c, double dt, const void *U_n, const double *lam_np1
     const void *X[4] = {U_n, X1, X2, X3};
     const bool sets = have_adjoint_sets(c);    // every stage state's split and traces kept
     if (sets) {
-        st = prepare_adjoint(c, U_n, adj_set(c, 0));
+        st = prepare_adjoint(c, U_n, adj_set(c, 0), true);
         if (st == DG_OK) st = stage_adjoint(c, U_n, U_n, X1, 0, 0.0, 1.0, 0.5 * dt);
         if (st == DG_OK) st = stage_adjoint(c, X1, X1, X2, 1, 0.0, 1.0, 0.5 * dt);
         if (st == DG_OK) st = stage_adjoint(c, X2, U_n, X3, 2, 2.0 / 3.0, 1.0 / 3.0, dt / 6.0);

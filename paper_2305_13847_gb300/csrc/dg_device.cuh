@@ -173,6 +173,7 @@ struct KArgs {
     // float64: the derived fields of the state produced (null: `derived`, in
     // place) and its rho_v (null: not stored; the adjoint kernels read it)
     Real *derived_out, *rv_out;
+    int fail_extra;   // times more that a failing node counts (a split that stands for several)
 };
 
 // float64 value of a storage-type value (widen: integer pipe)
@@ -1388,8 +1389,8 @@ __device__ __forceinline__ void derive_and_store(const KArgs<Real> &A, const Rea
     const size_t gi = (size_t)e * S::NP + a;
     const int lev = iz * S::P1 + digit<S::D, S::P1>(a, S::VERT);
     const NodeDerived nd = derive_node<S>(u, A, lev, Tprev);
-    if (!nd.conv) atomicAdd(&A.flags[0], 1ull);
-    if (!nd.phys) atomicAdd(&A.flags[1], 1ull);
+    if (!nd.conv) atomicAdd(&A.flags[0], 1ull + A.fail_extra);
+    if (!nd.phys) atomicAdd(&A.flags[1], 1ull + A.fail_extra);
     Real gm;
     if (sizeof(Real) == sizeof(float)) {
         T = (Real)nd.Tf;

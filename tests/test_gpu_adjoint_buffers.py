@@ -67,3 +67,22 @@ def test_adjoint_step_with_and_without_kept_states(dim, n, order):
         dm.dg_free(ctx)
     assert np.array_equal(a, c)
     assert np.all(np.linalg.norm(a - b, axis=1) <= 1e-12 * np.linalg.norm(a, axis=1))
+
+
+@pytest.mark.parametrize("keep", [0, 1])
+def test_adjoint_step_counts_do_not_depend_on_its_memory(keep):
+    """One overheated node (finite, above 1000 K) in each of the four stage states of a vanishing step:
+    counted twice per state, for the stage's split and the reversal's, whether the second is made or not."""
+    prob = _problem()
+    U = perturbed_state(prob, seed=45)
+    U[prob.i_E, 4, 5] = 2e6
+    ctx = library_context(prob)
+    try:
+        dm.dg_set_adjoint_memory(ctx, keep)
+        Ud = to_device(U, torch.float64)
+        out = torch.empty_like(Ud)
+        dm.dg_adjoint_step(ctx, 1e-12, Ud, torch.ones_like(Ud), out)
+        st, counts = dm.dg_check_status(ctx)
+        assert st == dm.DG_ENONPHYS and list(counts) == [0, 8]
+    finally:
+        dm.dg_free(ctx)
