@@ -541,7 +541,8 @@ def fp64_alu_roofline(info, w, t_total, steps, sm_count, sm_mhz, probe_tflops, h
            "algorithmic_flops_per_node": fpn,
            "flops_per_node_items": items, "avg_launch_ms": 1000.0 * launch_s,
            # the linear contractions run as fixed point on the integer pipe, beside
-           # the FP64 pipe, so frac may pass 1; this is the fraction of the rest
+           # the FP64 pipe, so frac may pass 1; this is the fraction of the rest,
+           # which the report takes (fp64_pipe_headline)
            "integer_pipe_items": list(INTEGER_PIPE_ITEMS),
            "frac_without_integer_items":
                achieved / peak * (1.0 - sum(items[k] for k in INTEGER_PIPE_ITEMS) / fpn),
@@ -549,6 +550,23 @@ def fp64_alu_roofline(info, w, t_total, steps, sm_count, sm_mhz, probe_tflops, h
                                        "algorithmic_bytes_per_launch")}}
     if probe_tflops:
         out["fp64_fma_probe"] = {"tflops": probe_tflops, "frac_of_probe": achieved / probe_tflops}
+    return out
+
+
+def fp64_pipe_headline(roof):
+    """The float64 roofline with achieved and frac over the items that run on
+    the FP64 pipe, whose rate the peak is: the linear contractions are integer
+    operations beside it.  All items together go to all_items, as a ratio
+    that may pass 1 and is no fraction of a peak."""
+    out = dict(roof)
+    share = out.pop("frac_without_integer_items") / out["frac"]
+    out["all_items"] = {"achieved": out["achieved"], "ratio_to_fp64_peak": out["frac"]}
+    out["achieved"] *= share
+    out["frac"] *= share
+    if "fp64_fma_probe" in out:
+        probe = dict(out["fp64_fma_probe"])
+        probe["frac_of_probe"] *= share
+        out["fp64_fma_probe"] = probe
     return out
 
 
@@ -813,7 +831,8 @@ def run_gb300(args):
         except Exception:
             probe = None
         sm_mhz = clocks.get("sm_mhz") or 2070.0
-        roof = fp64_alu_roofline(info, w, t_max, args.steps, sm_count, sm_mhz, probe, roof)
+        roof = fp64_pipe_headline(
+            fp64_alu_roofline(info, w, t_max, args.steps, sm_count, sm_mhz, probe, roof))
     dm.dg_free(ctx)
     del host
 
