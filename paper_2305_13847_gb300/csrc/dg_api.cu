@@ -354,9 +354,11 @@ int upload_and_prepare(dg_ctx *c, const void *host) {
 // The results are the same bits.  Small meshes under DG_FACES_AUTO go inline:
 // up to the lines below, the second launch and its latency cost more than the
 // doubled face work (us per step, inline against face pass; float64 2-D: 100
-// tiles 59 / 75, 160 tiles 132 / 108; 3-D: 96 tiles 126 / 116; FP32-bulk: 128
-// tiles 44 / 54, 512 tiles 58 / 74, 800 tiles 74 / 77, 1024 tiles 89 / 87).
-// The members of an ensemble share the chip, so their total work counts.
+// tiles 59 / 75, 160 tiles 132 / 108, the line at 101; FP32-bulk: 128 tiles
+// 44 / 54, 512 tiles 58 / 74, 800 tiles 74 / 77, 1024 tiles 89 / 87, the line
+// at 608; each from one order).  Float64 3-D: 96 tiles 126 / 116, always the
+// face pass; fewer tiles are not measured.  The members of an ensemble share
+// the chip, so their total work counts.
 bool use_face_pass(const dg_ctx *c) {
     if (!c->face_pass) return false;
     if (c->cfg.faces != DG_FACES_AUTO || c->diff || c->in_ensemble) return true;
@@ -573,6 +575,12 @@ void drop_adjoint_sets(dg_ctx *c) {
 // sets each state is split again, with the same result.
 bool have_adjoint_sets(dg_ctx *c) {
     if (c->adj_sets || c->adj_sets_off) return c->adj_sets != nullptr;
+    // a capture takes no allocation: this step splits again
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
     c->adj_sets_off = true;     // decided once
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t trace = up((size_t)2 * c->cfg.dim * c->ne * c->trace_face * sizeof(double));

@@ -86,3 +86,32 @@ def test_adjoint_step_counts_do_not_depend_on_its_memory(keep):
         assert st == dm.DG_ENONPHYS and list(counts) == [0, 8]
     finally:
         dm.dg_free(ctx)
+
+
+def test_adjoint_step_captured_before_its_first_use():
+    """A first reversed step inside a stream capture, after dg_rhs_adjoint has made the common scratch:
+    it allocates nothing, and a replay gives the eager step without kept states, bit by bit."""
+    prob = _problem()
+    U = to_device(perturbed_state(prob, seed=47), torch.float64)
+    g = torch.Generator().manual_seed(9)
+    lam = torch.randn(U.shape, generator=g, dtype=torch.float64).cuda()
+    a, b, r = (torch.empty_like(U) for _ in range(3))
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = library_context(prob, stream=stream)
+    try:
+        dm.dg_rhs_adjoint(ctx, U, lam, r)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(stream):
+            graph.capture_begin()
+            dm.dg_adjoint_step(ctx, 0.02, U, lam, a)
+            graph.capture_end()
+            graph.replay()
+        stream.synchronize()
+        dm.dg_set_adjoint_memory(ctx, 0)
+        dm.dg_adjoint_step(ctx, 0.02, U, lam, b)
+        stream.synchronize()
+        assert np.array_equal(a.cpu().numpy(), b.cpu().numpy())
+    finally:
+        dm.dg_free(ctx)
