@@ -85,9 +85,9 @@ struct MeshData {
     // faces normal to e_j: a grid of nfn[j] (= n_j, + 1 with walls) x the other n,
     // nfaces[j] of them; face c lies between the elements at coordinates c - 1
     // and c along e_j.  The face kernel covers direction j with fblk[j] CTAs
-    // and stores, per element, the outward flux of each of its faces
-    // (fbuf [ne][2D][NFP][NFP1], NFP = NF, or 2 NF with the diffusion's
-    // symmetry terms), so that a stage tile reads one contiguous block.
+    // and stores one block per face (FaceLayout: G along +e_j, with diffusion
+    // also the symmetry terms), face-major, which the two elements of the face
+    // read by index (ftab).
     int nfn[3];
     int nfaces[3];
     int fblk[3];

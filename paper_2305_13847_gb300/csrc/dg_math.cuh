@@ -170,6 +170,9 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
 
 __device__ __forceinline__ double sqrt_nr(double x) { return x > 0.0 ? x * rsqrt_nr(x) : 0.0; }
 
+// 2^k, -1023 < k < 1024
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
 // r^(-1/n) for 0 < r <= 2^100, n = 16 and 8 (the seed needs r below the
 // float32 maximum; the callers pass rain densities and density ratios, far
 // below 1): a float32 seed y (relative error delta
@@ -183,9 +186,6 @@ __device__ __forceinline__ double sqrt_nr(double x) { return x > 0.0 ? x * rsqrt
 // smallest subnormal is 2^-1074 > 2^-96 2^-1152); the loop stops there also
 // for r <= 0, which the callers exclude (the result is then not a number).
 // r > 0 orders like its bit pattern, so the test needs no float64 compare.
-// 2^k, -1023 < k < 1024
-__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
-
 constexpr double kTiny = 0x1p-96;
 constexpr double kUp = 0x1p128;
 
